@@ -220,15 +220,16 @@ void tc_shape(usr::ConvTcArgs& a, int n_out, int K, bool bf16, long long ctas_m)
     a.cols = (n_out + a.ntiles - 1) / a.ntiles;
     a.NT = ((a.cols + 1 + 15) / 16) * 16;
     a.tmem_cols = 32;
-    while (a.tmem_cols < a.NT) a.tmem_cols *= 2;
+    while (a.tmem_cols < 2 * a.NT) a.tmem_cols *= 2;     // two accumulators
     const int kstage = bf16 ? 64 : 32;
     const int nk = (K + kstage - 1) / kstage;
     const size_t stage = (size_t)(2 * 128 + 2 * a.NT) * 128;
     int S = (int)((200 * 1024) / stage);
     S = std::min(S, std::min(nk, 4));
     a.stages = std::max(1, std::min(S, usr::kConvTcMaxStages));
-    // keep (CTAs per SM) x (TMEM columns) <= 512 by padding the shared memory request
-    const size_t floor_smem = (size_t)228 * 1024 * a.tmem_cols / 512 + 1024;
+    // keep (CTAs per SM) x (TMEM columns) <= 512 by padding the shared memory request: one CTA more than that must
+    // not fit the SM's 228 KB (1 KB of which each CTA takes besides its request)
+    const size_t floor_smem = (size_t)228 * 1024 / (512 / a.tmem_cols + 1);
     a.smem = (int)std::max(usr::conv_tc_smem(a), floor_smem);
 }
 

@@ -266,7 +266,7 @@ struct ConvTcArgs {
     int n_out;              // output columns in all
     int nterms, nx, ny, nz;
     int stages;             // TMA ring depth
-    int tmem_cols;          // tensor-memory columns allocated (power of two >= NT)
+    int tmem_cols;          // tensor-memory columns allocated (power of two >= 2 NT: two accumulators)
     int smem;               // dynamic shared memory per CTA (bytes; padded so that the CTAs an SM
                             // can hold never ask for more than 512 TMEM columns together)
     const float* mu;        // per-term mean of the 1D kernel (passes 1, 2)
