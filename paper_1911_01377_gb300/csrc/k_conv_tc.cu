@@ -319,6 +319,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
         const int c_lo = tile * g.cols;
         float muj = 0.f;
         if (g.pass != 3) muj = g.mu[batch];
+        // the k = 0 mode of rho, dropped: a constant line adds nothing to the zero-mean part, K mean to the sum
+        if (g.pass == 1 && g.mean) dc -= (float)((double)g.K * *g.mean);
         int lx = 0, lz = 0;
         if (g.pass == 2) {
             lx = line / g.nz;

@@ -1,22 +1,8 @@
 /*
- * k_grid.cu -- the particle-grid legs of the far part (Sec. V with Gaussian
- * spreading, the GSE scheme named in Sec. IV.A), atomic-free and
- * deterministic.  Both grid kernels work on blocks of cells: one CTA owns
- * kb_x x kb_y x kb_z cells of the sorted cell list and a shared-memory tile of
- * grid points covering the P^3 stencils of all their atoms.
+ * k_grid.cu -- the gather leg of the far part (Sec. V with Gaussian spreading,
+ * the GSE scheme named in Sec. IV.A; the spreading leg is k_spread.cu) and the
+ * combination with the near part, atomic-free and deterministic.
  *
- *   spread   rho_g = sum_i q_i exp(-|g - r_i|^2 / (2 sigma_s^2)) (normalisation
- *            folded into the convolution scale).  The CTA's warps own disjoint
- *            sets of tile rows (y = warp mod 8) and every warp walks the
- *            block's atoms in sorted order, adding the stencil columns of its
- *            rows (one lane per column and group of planes) with plain
- *            shared-memory read-modify-writes: no atomics, and every tile point
- *            receives its terms in a fixed order.  The
- *            tile is stored whole to a tile buffer, and the block's tile sum
- *            is kept; the last CTA forms the grid mean (the k = 0 mode,
- *            dropped per Eq. 4) from those sums in block order.
- *   reduce   one thread per grid point adds the tiles that hold it, in block
- *            order, and subtracts the grid mean.
  *   gather   phi_far,i = sum_g w(g - r_i) psi_g and F_far,i = -q_i grad phi_far,i
  *            (the second spreading Gaussian of Eq. 32's 1/|S(k)|^2), per sorted
  *            atom, reading psi from global memory; contracts the stencil
@@ -25,8 +11,6 @@
  *            caller order, and E = 1/2 sum q_i phi_i and its parts
  *            (compensated FP32 within a warp, FP64 across warps and blocks).
  */
-#include <cuda_bf16.h>
-
 #include "usr_internal.h"
 
 namespace usr {
@@ -35,9 +19,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kChunk = 128;         // atoms whose weights are staged at once (spread)
-constexpr int kGChunk = 128;        // atoms staged at once (gather)
-constexpr int kMaxRows = 64;        // (cz, cy) rows of cells per block
 
 __device__ __forceinline__ double warp_sum_d(double v)
 {
@@ -97,271 +78,7 @@ __device__ __forceinline__ int wrap_once(int v, int n)
     return v;
 }
 
-/* Block coordinates, cell range and tile origin of CTA `bid`. */
-struct BlockGeom {
-    int c0[3], c1[3];
-    int o[3];
-};
-
-__device__ __forceinline__ BlockGeom block_geom(const GridArgs& g, int bid)
-{
-    BlockGeom b;
-    const int nb0 = g.tg.nbk[0], nb1 = g.tg.nbk[1];
-    const int bc[3] = {bid % nb0, (bid / nb0) % nb1, bid / (nb0 * nb1)};
-    #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        b.c0[a] = bc[a] * g.tg.kb[a];
-        b.c1[a] = min(g.box.nc[a], b.c0[a] + g.tg.kb[a]);
-        b.o[a] = g.tab.org[a][bc[a]];
-    }
-    return b;
-}
-
-/*
- * The block's atoms are the x-runs of its (cz, cy) cell rows, contiguous in
- * the sorted array.  Fills rs/pre (row start, prefix count) and returns the
- * total.  Called by all threads; thread 0 writes, then a barrier.
- */
-__device__ int block_rows(const GridArgs& g, const BlockGeom& bg, const int* __restrict__ cell_start, int* rs,
-                          int* pre)
-{
-    const int ncx = g.box.nc[0], ncy = g.box.nc[1];
-    const int ny = bg.c1[1] - bg.c0[1];
-    const int nrows = ny * (bg.c1[2] - bg.c0[2]);
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int r = 0; r < nrows; ++r) {
-            const int cz = bg.c0[2] + r / ny, cy = bg.c0[1] + r % ny;
-            const int row = (cz * ncy + cy) * ncx;
-            const int s = cell_start[row + bg.c0[0]], e = cell_start[row + bg.c1[0]];
-            rs[r] = s;
-            pre[r] = acc;
-            acc += e - s;
-        }
-        pre[nrows] = acc;
-    }
-    __syncthreads();
-    return pre[nrows];
-}
-
-/* Sorted-array index of the block's j-th atom. */
-__device__ __forceinline__ int block_atom(int j, const int* rs, const int* pre)
-{
-    int r = 0;
-    while (pre[r + 1] <= j) ++r;
-    return rs[r] + (j - pre[r]);
-}
-
 }  // namespace
-
-/* ------------------------------------------------------------------ spread */
-
-template <int P>
-__global__ void __launch_bounds__(kThreads, 2) k_spread(const float4* __restrict__ pos,
-                                                        const int* __restrict__ cell_start, GridArgs g,
-                                                        float* __restrict__ tilebuf, double* __restrict__ partial,
-                                                        unsigned int* __restrict__ counter,
-                                                        double* __restrict__ mean, int* __restrict__ status)
-{
-    pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
-    constexpr int H = P / 2;
-    static_assert(P <= 2 * kWarps && P <= 32, "at most two stencil rows per warp");
-    extern __shared__ float4 smem4[];
-    float* tile = reinterpret_cast<float*>(smem4);
-    constexpr int PA = (P + 3) & ~3;              // weight rows padded to 16 bytes
-    __shared__ __align__(16) float W[kChunk][3][PA];
-    __shared__ int B[kChunk][3];
-    __shared__ int2 R[kChunk];                    // (tile offset of the stencil corner or -1, its y)
-    __shared__ float4 sp[kChunk];
-    __shared__ int rs[kMaxRows], pre[kMaxRows + 1];
-    __shared__ double red[kWarps];
-    __shared__ int is_last;
-
-    const int Tx = g.tg.T[0], Ty = g.tg.T[1], Tz = g.tg.T[2];
-    const int TT = Tx * Ty * Tz;
-    const int TXY = Tx * Ty;
-    const int PS = g.tg.ps;                       // plane stride in shared memory (>= TXY, bank-conflict free)
-    const BlockGeom bg = block_geom(g, blockIdx.x);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    {
-        float4* t4 = smem4;
-        for (int t = threadIdx.x; t < ((PS * Tz) >> 2); t += kThreads) t4[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const int natoms = block_rows(g, bg, cell_start, rs, pre);   // contains a barrier
-
-    for (int c0 = 0; c0 < natoms; c0 += kChunk) {
-        const int nch = min(kChunk, natoms - c0);
-        // phase 1: stage the chunk's positions, then per-atom 1D weights (q folded
-        // into the x weights) and tile base
-        for (int a = threadIdx.x; a < nch; a += kThreads) {
-            const int s = block_atom(c0 + a, rs, pre);
-            sp[a] = USR_IN_BOUNDS(s, g.max_atoms, status) ? pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < nch * 3 * P; idx += kThreads) {
-            const int a = idx / (3 * P), rem = idx - a * 3 * P;
-            const int ax = rem / P, k = rem - ax * P;
-            const float4 p = sp[a];
-            // per-axis constants selected without dynamic indexing (keeps them in registers)
-            const float pc = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
-            const float gs = ax == 0 ? g.box.gs[0] : (ax == 1 ? g.box.gs[1] : g.box.gs[2]);
-            const float hh = ax == 0 ? g.hh[0] : (ax == 1 ? g.hh[1] : g.hh[2]);
-            const int org = ax == 0 ? bg.o[0] : (ax == 1 ? bg.o[1] : bg.o[2]);
-            const int Ta = ax == 0 ? Tx : (ax == 1 ? Ty : Tz);
-            const float u = pc * gs;
-            const float f = floorf(u);
-            const float t = u - f;
-            const float d = (float)(k - H + 1) - t;
-            float w = __expf(-d * d * hh);
-            if (ax == 0) w *= p.w;
-            W[a][ax][k] = w;
-            if (k == 0) {
-                const int base = (int)f - H + 1 - org;
-                const bool ok = base >= 0 && base + P <= Ta;
-                B[a][ax] = ok ? base : -1;
-                if (!ok) atomicOr(status, 2);    // cannot happen for wrapped positions
-            }
-        }
-        __syncthreads();
-        // phase 1b: one record per atom, the tile offset of its stencil corner (or -1) and its y
-        for (int a = threadIdx.x; a < nch; a += kThreads) {
-            const int bx = B[a][0], by = B[a][1], bz = B[a][2];
-            R[a] = make_int2(bx < 0 || by < 0 || bz < 0 ? -1 : bz * PS + by * Tx + bx, by);
-        }
-        __syncthreads();
-        // phase 2: warp w owns the tile rows ty = w (mod 8); for each atom it adds
-        // the stencil columns of its one or two rows.  Lane = (column jx, group of
-        // planes): P columns x G groups, each lane updating PG consecutive planes.
-        {
-            constexpr int G = 32 / P;                  // plane groups per row
-            constexpr int PG = (P + G - 1) / G;        // planes per lane
-            static_assert((kWarps & (kWarps - 1)) == 0, "row ownership by a mask");
-            const int jx = lane % P, grp = lane / P;
-            const int k0 = grp * PG;
-            float* const tl = tile + k0 * PS + jx;
-            for (int a = 0; a < nch; ++a) {
-                const int2 r = R[a];
-                if (r.x < 0 || grp >= G) continue;
-                float wz[PG];
-                #pragma unroll
-                for (int k = 0; k < PG; ++k) wz[k] = (k0 + k < P) ? W[a][2][k0 + k] : 0.f;
-                const float wxa = W[a][0][jx];
-                for (int jy = (warp - r.y) & (kWarps - 1); jy < P; jy += kWarps) {
-                    const float v = wxa * W[a][1][jy];
-                    float* col = tl + r.x + jy * Tx;
-                    float t[PG];
-                    #pragma unroll
-                    for (int k = 0; k < PG; ++k)
-                        if (k0 + k < P) t[k] = col[k * PS];
-                    #pragma unroll
-                    for (int k = 0; k < PG; ++k)
-                        if (k0 + k < P) col[k * PS] = fmaf(v, wz[k], t[k]);
-                }
-            }
-        }
-        __syncthreads();
-    }
-
-    // store the tile, sum it in a fixed order
-    double local;
-    {
-        const float4* t4 = smem4;
-        float4* out4 = reinterpret_cast<float4*>(tilebuf + (size_t)blockIdx.x * TT);
-        CSum cs;
-        const int pq = TXY >> 2;                  // float4s per plane (TXY is a multiple of 4)
-        for (int t = threadIdx.x; t < (TT >> 2); t += kThreads) {
-            const int z = t / pq;
-            const float4 v = t4[z * (PS >> 2) + (t - z * pq)];   // dense in the tile buffer
-            out4[t] = v;
-            cs.add(v.x);
-            cs.add(v.y);
-            cs.add(v.z);
-            cs.add(v.w);
-        }
-        local = warp_sum_c(cs);
-    }
-    if (lane == 0) red[warp] = local;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += red[w];
-        partial[blockIdx.x] = s;
-        __threadfence();
-        const unsigned int ticket = atomicAdd(counter, 1u);
-        is_last = (ticket == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (is_last) {
-        // grid mean from the block sums, in block order (the same whichever CTA is last)
-        __threadfence();
-        double s = 0.0;
-        for (int k = threadIdx.x; k < (int)gridDim.x; k += kThreads) s += ((volatile double*)partial)[k];
-        s = warp_sum_d(s);
-        if (lane == 0) red[warp] = s;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double tot = 0.0;
-            for (int w = 0; w < kWarps; ++w) tot += red[w];
-            *mean = tot / ((double)g.box.n[0] * g.box.n[1] * g.box.n[2]);
-            *counter = 0u;
-        }
-    }
-}
-
-/*
- * rho_g = (sum of the tiles holding g, in block order) - mean.  SPLIT = 0
- * writes FP32 rho; 1 and 2 write the operand split of the tensor-core
- * convolution instead: rho = hi + lo with hi rounded to TF32 (1) or BF16 (2).
- */
-template <int SPLIT>
-__global__ void __launch_bounds__(256) k_tile_reduce(GridArgs g, const float* __restrict__ tilebuf,
-                                                     const double* __restrict__ mean, void* __restrict__ rho,
-                                                     void* __restrict__ rho_lo, float* __restrict__ rho32,
-                                                     int* __restrict__ status)
-{
-    pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
-    // grid: x over the (y, x) plane in blocks of 256, y over z (32-bit index arithmetic)
-    const int n0 = g.box.n[0], n1 = g.box.n[1];
-    const int pxy = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pxy >= n0 * n1) return;
-    const int y = pxy / n0, x = pxy - y * n0, z = blockIdx.y;
-    const long long idx = (long long)z * n0 * n1 + pxy;
-    const int T0 = g.tg.T[0], T1 = g.tg.T[1], T2 = g.tg.T[2];
-    const long long TT = (long long)T0 * T1 * T2;
-    const int nb0 = g.tg.nbk[0], nb1 = g.tg.nbk[1];
-    const int cz = g.tab.red_cnt[2][z], cy = g.tab.red_cnt[1][y], cx = g.tab.red_cnt[0][x];
-    const int2* pz = g.tab.red_pair[2] + (size_t)z * g.tg.rmax[2];
-    const int2* py = g.tab.red_pair[1] + (size_t)y * g.tg.rmax[1];
-    const int2* px = g.tab.red_pair[0] + (size_t)x * g.tg.rmax[0];
-    float s = 0.f;
-    for (int iz = 0; iz < cz; ++iz) {
-        const int2 bz = pz[iz];
-        for (int iy = 0; iy < cy; ++iy) {
-            const int2 by = py[iy];
-            const long long rowbase = ((long long)(bz.x * nb1 + by.x) * nb0) * TT + ((long long)bz.y * T1 + by.y) * T0;
-            for (int ix = 0; ix < cx; ++ix) {
-                const int2 bx = px[ix];
-                const long long t = rowbase + (long long)bx.x * TT + bx.y;
-                if (USR_IN_BOUNDS(t, (long long)nb0 * nb1 * g.tg.nbk[2] * TT, status)) s += __ldg(tilebuf + t);
-            }
-        }
-    }
-    const float v = s - (float)*mean;
-    if (SPLIT != 0 && rho32) rho32[idx] = v;     // FP32 copy for the virial convolutions
-    if (SPLIT == 0) {
-        static_cast<float*>(rho)[idx] = v;
-    } else if (SPLIT == 1) {
-        uint32_t hb;
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hb) : "f"(v));
-        const float h = __uint_as_float(hb);
-        static_cast<float*>(rho)[idx] = h;
-        static_cast<float*>(rho_lo)[idx] = v - h;
-    } else {
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        static_cast<__nv_bfloat16*>(rho)[idx] = h;
-        static_cast<__nv_bfloat16*>(rho_lo)[idx] = __float2bfloat16_rn(v - __bfloat162float(h));
-    }
-}
 
 /*
  * Grid mean of psi.  Exact arithmetic gives psi no k = 0 mode (rho has its
@@ -513,7 +230,7 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
         for (int a = 0; a < 3; ++a) {
             const float uu = pc[a] * g.box.gs[a];
             const float f = floorf(uu);
-            tt[a] = uu - f;
+            tt[a] = grid_frac(g.box, a, pc[a], f);
             base[a] = (int)f - H + 1;
         }
         float wz[P], dz[P], wx[NC], dx[NC];
@@ -698,59 +415,9 @@ __global__ void __launch_bounds__(kThreads) k_combine(int n, const float4* __res
 
 /* ------------------------------------------------------------------ launch */
 
-int tile_blocks(const TileGeom& tg) { return tg.nbk[0] * tg.nbk[1] * tg.nbk[2]; }
-
-size_t tile_floats(const TileGeom& tg) { return (size_t)tg.T[0] * tg.T[1] * tg.T[2]; }
-
-template <int P>
-static void set_smem(size_t bytes)
-{
-    cudaFuncSetAttribute(k_spread<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-/* Allow every stencil variant the largest tile a plan may choose. */
-usr_status grid_kernel_setup(size_t bytes)
-{
-    set_smem<8>(bytes);
-    set_smem<10>(bytes);
-    set_smem<12>(bytes);
-    set_smem<14>(bytes);
-    set_smem<16>(bytes);
-    return cudaGetLastError() == cudaSuccess ? USR_OK : USR_ERR_CUDA;
-}
-
-#define USR_SPREAD_CASE(PP)                                                                                     \
-    case PP:                                                                                                    \
-        launch_pdl(k_spread<PP>, nb, kThreads, smem, st, spos, cell_start, g, tilebuf, partial, counter, mean, \
-                   status);                                                                                     \
-        break;
-
-void launch_spread(int P, const float4* spos, const int* cell_start, const GridArgs& g, float* tilebuf, int split,
-                   void* rho, void* rho_lo, double* partial, unsigned int* counter, double* mean, int* status,
-                   cudaStream_t st, float* rho32)
-{
-    const int nb = tile_blocks(g.tg);
-    const size_t smem = sizeof(float) * (size_t)g.tg.ps * g.tg.T[2];
-    switch (P) {
-        USR_SPREAD_CASE(8)
-        USR_SPREAD_CASE(10)
-        USR_SPREAD_CASE(12)
-        USR_SPREAD_CASE(14)
-        default:
-        USR_SPREAD_CASE(16)
-    }
-    const dim3 nr((unsigned)((g.box.n[0] * g.box.n[1] + 255) / 256), (unsigned)g.box.n[2]);
-    if (split == 1)
-        launch_pdl(k_tile_reduce<1>, nr, 256, 0, st, g, tilebuf, mean, rho, rho_lo, rho32, status);
-    else if (split == 2)
-        launch_pdl(k_tile_reduce<2>, nr, 256, 0, st, g, tilebuf, mean, rho, rho_lo, rho32, status);
-    else
-        launch_pdl(k_tile_reduce<0>, nr, 256, 0, st, g, tilebuf, mean, rho, nullptr, nullptr, status);
-}
-
 #define USR_GATHER_CASE(PP)                                                                \
     case PP:                                                                               \
-        launch_pdl(k_gather<PP>, nb, kGThreads, 0, st, spos, n, psi, g, far4, partial, counter, psi_mean, status); \
+        launch_with(-1, k_gather<PP>, nb, kGThreads, 0, st, spos, n, psi, g, far4, partial, counter, psi_mean, status); \
         break;
 
 static int gather_blocks(int n, int P)

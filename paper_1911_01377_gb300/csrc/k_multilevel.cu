@@ -58,11 +58,11 @@ __device__ __forceinline__ long long offs(int col, int g, int b, int d0, int d1,
 
 /*
  * Stage rows [g0, g0 + ROWS) (periodic in n_in) of 32 columns starting at col0 into S[row][col].  Columns
- * past ncol read as zero.  All of a thread's loads are issued before its shared-memory stores.
+ * past ncol read as zero; `less` (AX = 0) is taken off every value.  All of a thread's loads are issued before its shared-memory stores.
  */
 template <int AX, int ROWS>
 __device__ __forceinline__ void stage(float (*S)[kMlPad], const float* __restrict__ in, int g0, int n_in,
-                                      int col0, int ncol, int b, int d0, int d1)
+                                      int col0, int ncol, int b, int d0, int d1, float less = 0.f)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (AX == 0) {
@@ -76,7 +76,7 @@ __device__ __forceinline__ void stage(float (*S)[kMlPad], const float* __restric
             #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 const int r = lane + 32 * k;
-                v[li][k] = ok && r < ROWS ? in[offs<0>(col0 + l, wrap(g0 + r, n_in), b, d0, d1, n_in)] : 0.f;
+                v[li][k] = ok && r < ROWS ? in[offs<0>(col0 + l, wrap(g0 + r, n_in), b, d0, d1, n_in)] - less : 0.f;
             }
         }
         #pragma unroll
@@ -136,8 +136,8 @@ __device__ __forceinline__ void emit(float (*S)[kMlPad], const float acc[4], flo
 
 /* CTA coordinates: blockIdx.x = column tile, blockIdx.y = output tile along AX, blockIdx.z = batch index. */
 template <int AX, int OUT>
-__global__ void __launch_bounds__(256) k_ml_restrict(const float* __restrict__ in, float* __restrict__ out,
-                                                     float* __restrict__ out_lo, int d0, int d1, int ncol,
+__global__ void __launch_bounds__(256) k_ml_restrict(const float* __restrict__ in, const double* __restrict__ mean,
+                                                     float* __restrict__ out, float* __restrict__ out_lo, int d0, int d1, int ncol,
                                                      int n_in, MlTaps taps, long long out_elems, int* status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) k_ml_restrict(const float* __restrict__ i
     const int n_out = n_in / 2;
     const int col0 = blockIdx.x * 32, a0 = blockIdx.y * kMlCh, b = blockIdx.z;
     // outputs a0 .. a0 + 31 read fine rows 2 a0 - T .. 2 (a0 + 31) + T
-    stage<AX, kMlWinR>(S, in, 2 * a0 - kMlT, n_in, col0, ncol, b, d0, d1);
+    stage<AX, kMlWinR>(S, in, 2 * a0 - kMlT, n_in, col0, ncol, b, d0, d1, AX == 0 ? (float)*mean : 0.f);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -205,14 +205,14 @@ void shape(const int* od, dim3* grid, int* ncol)
 }
 
 template <int AX, int OUT>
-void restrict_axis(const float* in, float* out, float* out_lo, const int* od, const MlTaps& w, int* status,
+void restrict_axis(const float* in, const double* mean, float* out, float* out_lo, const int* od, const MlTaps& w, int* status,
                    cudaStream_t st)
 {
     dim3 g;
     int ncol;
     shape<AX>(od, &g, &ncol);
     const long long elems = (long long)od[0] * od[1] * od[2];
-    launch_pdl(k_ml_restrict<AX, OUT>, g, 256, 0, st, in, out, out_lo, od[0], od[1], ncol, 2 * od[AX], w, elems,
+    launch_pdl(k_ml_restrict<AX, OUT>, g, 256, 0, st, in, mean, out, out_lo, od[0], od[1], ncol, 2 * od[AX], w, elems,
                status);
 }
 
@@ -228,18 +228,18 @@ void prolong_axis(const float* in, float* out, const int* od, const MlTaps& w, i
 
 }  // namespace
 
-void launch_ml_restrict(const MlArgs& m, const float* rho, float* t1, float* t2, float* rho_c, float* rho_c_lo,
+void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c, float* rho_c_lo,
                         int* status, cudaStream_t st)
 {
     const int d1[3] = {m.nc[0], m.n[1], m.n[2]};
     const int d2[3] = {m.nc[0], m.nc[1], m.n[2]};
     const int d3[3] = {m.nc[0], m.nc[1], m.nc[2]};
-    restrict_axis<0, 0>(rho, t1, nullptr, d1, m.taps, status, st);
-    restrict_axis<1, 0>(t1, t2, nullptr, d2, m.taps, status, st);
+    restrict_axis<0, 0>(rho, mean, t1, nullptr, d1, m.taps, status, st);
+    restrict_axis<1, 0>(t1, nullptr, t2, nullptr, d2, m.taps, status, st);
     if (rho_c_lo)
-        restrict_axis<2, 1>(t2, rho_c, rho_c_lo, d3, m.taps, status, st);
+        restrict_axis<2, 1>(t2, nullptr, rho_c, rho_c_lo, d3, m.taps, status, st);
     else
-        restrict_axis<2, 0>(t2, rho_c, nullptr, d3, m.taps, status, st);
+        restrict_axis<2, 0>(t2, nullptr, rho_c, nullptr, d3, m.taps, status, st);
 }
 
 void launch_ml_prolong(const MlArgs& m, const float* psi_c, float* t1, float* t2, float* psi, int* status,

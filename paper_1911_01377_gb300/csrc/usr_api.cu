@@ -81,9 +81,6 @@ struct usr_ctx {
     double* d_netq = nullptr;            // net charge of the last evaluation (FP64)
     unsigned int* d_counters = nullptr;
     double* d_psi_mean = nullptr;
-    // spreading tiles and the per-axis tile tables
-    float* d_tilebuf = nullptr;
-    int* d_tab[3] = {nullptr, nullptr, nullptr};
     // tensor-core convolutions: the fine grid's (TF32x3 or BF16x3) and, with the multilevel form, the coarse
     // grid's (TF32x3)
     bool tc = false, tc_bf16 = false;
@@ -152,8 +149,8 @@ void free_all(usr_ctx* c)
                     c->d_pstart, c->d_cidx, c->d_ccell, c->d_cpos, c->d_bblo, c->d_bbhi,
                     c->d_wpos, c->d_spos, c->d_nacc, c->d_gfull, c->d_gpart, c->d_gfirst, c->d_queue, c->d_rho, c->d_X, c->d_Y, c->d_psi, c->d_Bx, c->d_Ay,
                     c->d_Az, c->d_wx, c->d_wy, c->d_wz, c->d_spread_partial, c->d_mean, c->d_gather_partial,
-                    c->d_energy, c->d_netq, c->d_counters, c->d_in, c->d_out, c->d_near_dbg, c->d_far_dbg, c->d_far4, c->d_tilebuf,
-                    c->d_tab[0], c->d_tab[1], c->d_tab[2], c->d_psi_mean, c->d_ktab};
+                    c->d_energy, c->d_netq, c->d_counters, c->d_in, c->d_out, c->d_near_dbg, c->d_far_dbg, c->d_far4,
+                    c->d_psi_mean, c->d_ktab};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (TcConv* t : {&c->tcf, &c->tcc}) {
@@ -195,15 +192,10 @@ void fill_box(const Plan& P, usr::BoxF& b)
         b.invL[a] = (float)(1.0 / P.L[a]);
         b.cs[a] = (float)((double)P.cells[a] / P.L[a]);
         b.gs[a] = (float)((double)P.n[a] / P.L[a]);
+        b.gl[a] = (float)((double)P.n[a] / P.L[a] - (double)b.gs[a]);
         b.nc[a] = P.cells[a];
         b.n[a] = P.n[a];
     }
-}
-
-size_t tab_ints(const Plan& P, int a)
-{
-    const size_t head = (P.tile_org[a].size() + P.red_cnt[a].size() + 1) / 2 * 2;
-    return head + P.red_pair[a].size();
 }
 
 /*
@@ -279,7 +271,7 @@ double usr::plan_device_bytes(const Plan& P)
     const double ncell = (double)P.cells[0] * P.cells[1] * P.cells[2];
     const double G = (double)P.n[0] * P.n[1] * P.n[2], N = P.N;
     const double nx = P.n[0], ny = P.n[1], nz = P.n[2];
-    const double nsb = tile_blocks(P.tile);
+    const double nsb = spread_ctas(P.n);
     const double ncl = std::floor((na + 7 * ncell + 7) / 8);
     const double nmax = std::max(nx, std::max(ny, nz));
     double b = 4096 + 4 * (ncell + 1) * 3 + 16 * ncl * 8 + 4 * ncl * 8 + 4 * ncl + 32 * ncl;   // cells, clusters
@@ -287,8 +279,7 @@ double usr::plan_device_bytes(const Plan& P)
     b += na * (4 * 4 + 16 * 7 + 32);                                               // per-atom arrays
     const double ngr = near_max_groups((int)na, (int)ncell);
     b += 8 * (ncell + 1) + 4 * ngr + 4;                                            // pair-kernel groups
-    b += 4 * G + 8 * (nsb + kGatherBlocks + 4 * kCombineBlocks) + 8 * 11 + 4 * nsb * tile_floats(P.tile);
-    for (int a = 0; a < 3; ++a) b += 4.0 * ((P.tile_org[a].size() + P.red_cnt[a].size() + 1) / 2 * 2 + P.red_pair[a].size());
+    b += 4 * G + 8 * (nsb + kGatherBlocks + 4 * kCombineBlocks) + 8 * 11;
     if (P.p.virial) {   // six FP32 table sets, their inputs, two FP32 grids, warp slots, FP32 scratch grids
         b += 6 * 4 * N * (nx * nx + ny * ny + nz * nz + nx + ny + nz) + 6 * 8 * (3 * N * nmax + 4 * N);
         b += 8 * G + 48 * near_units((int)ngr) + 8 * (16 + kGridMeanBlocks);
@@ -429,7 +420,7 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     const size_t na = (size_t)(c->max_atoms > 0 ? c->max_atoms : 1);
     const size_t N = (size_t)P.N, G = (size_t)c->G;
     const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-    const int nsb = usr::tile_blocks(P.tile);
+    const int nsb = usr::spread_ctas(P.n);
     c->max_clusters = (int)((na + 7 * (size_t)c->ncell + 7) / 8);
     c->max_groups = usr::near_max_groups((int)na, c->ncell);
     const size_t ncl = (size_t)c->max_clusters;
@@ -471,8 +462,6 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     ENSURE(c->d_out, f4 * na);
     ENSURE(c->d_near_dbg, f4 * na);
     ENSURE(c->d_far_dbg, f4 * na);
-    ENSURE(c->d_tilebuf, fl * nsb * usr::tile_floats(P.tile));
-    for (int a = 0; a < 3; ++a) ENSURE(c->d_tab[a], i4 * tab_ints(P, a));
     Staged up;
     c->vir = p->virial != 0;
     c->vir_valid = false;
@@ -508,7 +497,7 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     if (c->vir) {
         ENSURE(c->d_vktab, db * nkt * 6);
         ENSURE(c->d_psiv, fl * G);
-        if (c->tc) ENSURE(c->d_rho32, fl * G);
+        ENSURE(c->d_rho32, fl * G);
         ENSURE(c->d_vnear, db * 6 * usr::near_units(c->max_groups));
         ENSURE(c->d_vdot, db * 6);
         ENSURE(c->d_vpart, db * usr::kGridMeanBlocks);
@@ -603,20 +592,6 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     tab.mu = c->d_ktab + 3 * N * nmax;
     tab.scale = c->d_ktab + 3 * N * nmax + 3 * N;
     fill_args(c);
-    // per axis: tile origins, then reduction counts, then (block, offset) pairs
-    for (int a = 0; a < 3; ++a) {
-        std::vector<int> t;
-        t.insert(t.end(), P.tile_org[a].begin(), P.tile_org[a].end());
-        t.insert(t.end(), P.red_cnt[a].begin(), P.red_cnt[a].end());
-        while (t.size() % 2) t.push_back(0);
-        t.insert(t.end(), P.red_pair[a].begin(), P.red_pair[a].end());
-        up.add(c->d_tab[a], t.data(), t.size());
-        const size_t off_cnt = P.tile_org[a].size();
-        const size_t off_pair = (off_cnt + P.red_cnt[a].size() + 1) / 2 * 2;
-        c->grid.tab.org[a] = c->d_tab[a];
-        c->grid.tab.red_cnt[a] = c->d_tab[a] + off_cnt;
-        c->grid.tab.red_pair[a] = reinterpret_cast<const int2*>(c->d_tab[a] + off_pair);
-    }
     c->grid.psi_mean = c->d_psi_mean;
     if (c->tc) {
         std::vector<float> mu(2 * N);
@@ -625,6 +600,7 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
             mu[N + j] = (float)P.mu[1][j];
         }
         if ((s = setup_tc(c, c->tcf, c->tc_bf16, (int)N, nx, ny, nz, mu, c->d_psi, up)) != USR_OK) return s;
+        c->tcf.targs[0].mean = c->d_mean;    // the coarse grid's rho has no mean: the restriction took it off
     }
     if (c->ml_tc) {
         const int Nc = P.Nc;
@@ -730,7 +706,6 @@ void fill_args(usr_ctx* c)
     g.F0 = (float)P.F0;
     g.F0d = P.F0;
     g.wsum = (float)P.wsum;
-    g.tg = P.tile;
 }
 
 usr_status check_device(const usr_ctx* c)
@@ -780,7 +755,8 @@ usr::ClusterList cluster_list(const usr_ctx* c)
 /* The evaluation sequence; xyzq/out are device pointers already checked. */
 /*
  * The three FP32 convolution passes of Sec. V on rho with the tables
- * {Bx, Ay, Az, wx, wy, wz} into psi (X and Y are the context's scratch); after
+ * {Bx, Ay, Az, wx, wy, wz} into psi (X and Y are the context's scratch), less the convolution of
+ * rho's grid mean (null: rho has none); after
  * each pass `after(k)` is called (stage marks).
  */
 struct Conv3 {
@@ -789,7 +765,7 @@ struct Conv3 {
 };
 
 template <typename F>
-void conv3(const Conv3& d, const float* rho, float* const* t, float* psi, cudaStream_t st, F after)
+void conv3(const Conv3& d, const float* rho, const double* mean, float* const* t, float* psi, cudaStream_t st, F after)
 {
     const int N = d.N, nx = d.nx, ny = d.ny, nz = d.nz;
     const long long G = (long long)nx * ny * nz;
@@ -800,7 +776,7 @@ void conv3(const Conv3& d, const float* rho, float* const* t, float* psi, cudaSt
         g.B = t[0]; g.ldb = (long long)N * nx;
         g.C = d.X; g.ldc = nx;
         g.nb2 = 1; g.nsplit = nx; g.c_split = G;
-        g.mode = 1; g.dcw = t[3]; g.mean = nullptr;   // rho has its mean removed already
+        g.mode = 1; g.dcw = t[3]; g.mean = mean;
         usr::launch_conv(g, 1, st);
     }
     after(0);
@@ -829,10 +805,10 @@ void conv3(const Conv3& d, const float* rho, float* const* t, float* psi, cudaSt
 }
 
 template <typename F>
-void fp32_conv(usr_ctx* c, const float* rho, float* const* t, float* psi, cudaStream_t st, F after)
+void fp32_conv(usr_ctx* c, const float* rho, const double* mean, float* const* t, float* psi, cudaStream_t st, F after)
 {
     const Plan& P = c->plan;
-    conv3(Conv3{P.N, P.n[0], P.n[1], P.n[2], c->d_X, c->d_Y}, rho, t, psi, st, after);
+    conv3(Conv3{P.N, P.n[0], P.n[1], P.n[2], c->d_X, c->d_Y}, rho, mean, t, psi, st, after);
 }
 
 /* The evaluation sequence; xyzq/out are device pointers already checked. */
@@ -879,19 +855,21 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
         NvtxRange r("usr: far chain (spread, convolutions, psi mean)");
         mark(3, sd);
         if (c->tc)
-            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, c->d_tilebuf, c->tc_bf16 ? 2 : 1,
-                               c->tcf.rho_hi, c->tcf.rho_lo, c->d_spread_partial, c->d_counters, c->d_mean, c->d_status,
-                               sd, (c->vir || c->mlN > 0) ? c->d_rho32 : nullptr);
+            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, c->tc_bf16 ? 2 : 1, c->tcf.rho_hi,
+                               c->tcf.rho_lo, (c->vir || c->mlN > 0) ? c->d_rho32 : nullptr, c->d_spread_partial,
+                               c->d_counters, c->d_mean, c->d_status, sd);
         else
-            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, c->d_tilebuf, 0, c->d_rho, nullptr,
+            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, 0, c->d_rho, nullptr, nullptr,
                                c->d_spread_partial, c->d_counters, c->d_mean, c->d_status, sd);
+        // the virial's grid products take FP32 rho without its mean; every other reader takes the mean off itself
+        if (c->vir) usr::launch_sub_mean(c->G, c->tc ? c->d_rho32 : c->d_rho, c->d_rho32, c->d_mean, sd);
         mark(4, sd);
         if (c->tc) {
             run_tc(c->tcf, c->inject_timeout, sd, [&](int k) { mark(5 + k, sd); });
             c->inject_timeout = false;
         } else {
             float* const t[6] = {c->d_Bx, c->d_Ay, c->d_Az, c->d_wx, c->d_wy, c->d_wz};
-            fp32_conv(c, c->d_rho, t, c->d_psi, sd, [&](int k) { mark(5 + k, sd); });
+            fp32_conv(c, c->d_rho, c->d_mean, t, c->d_psi, sd, [&](int k) { mark(5 + k, sd); });
         }
         if (c->mlN > 0) {
             // the wide terms on the coarse grid, added to psi (Sec. V, multilevel)
@@ -902,15 +880,15 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
             float* pc = ml_psi_c(c);
             const float* rho = c->tc ? c->d_rho32 : c->d_rho;
             if (c->ml_tc) {
-                usr::launch_ml_restrict(c->ml, rho, t1, t2, static_cast<float*>(c->tcc.rho_hi),
+                usr::launch_ml_restrict(c->ml, rho, c->d_mean, t1, t2, static_cast<float*>(c->tcc.rho_hi),
                                         static_cast<float*>(c->tcc.rho_lo), c->d_status, sd);
                 run_tc(c->tcc, false, sd, [](int) {});
             } else {
                 float* rc = t2 + c->ml_t2;
                 float* Xc = rc + Gc;
                 float* Yc = Xc + (size_t)c->mlN * Gc;
-                usr::launch_ml_restrict(c->ml, rho, t1, t2, rc, nullptr, c->d_status, sd);
-                conv3(Conv3{c->mlN, Q.nc[0], Q.nc[1], Q.nc[2], Xc, Yc}, rc, c->d_ctab, pc, sd, [](int) {});
+                usr::launch_ml_restrict(c->ml, rho, c->d_mean, t1, t2, rc, nullptr, c->d_status, sd);
+                conv3(Conv3{c->mlN, Q.nc[0], Q.nc[1], Q.nc[2], Xc, Yc}, rc, nullptr, c->d_ctab, pc, sd, [](int) {});
             }
             usr::launch_ml_prolong(c->ml, pc, t1, t2, c->d_psi, c->d_status, sd);
         }
@@ -940,9 +918,9 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
     if (c->vir) {
         NvtxRange r("usr: virial");
         // far virial: 1/2 <rho, psi_ab> per strain component, then the finalisation with E_far
-        const float* rho = c->tc ? c->d_rho32 : c->d_rho;
+        const float* rho = c->d_rho32;
         for (int cmp = 0; cmp < 6; ++cmp) {
-            fp32_conv(c, rho, c->d_vtab[cmp], c->d_psiv, st, [](int) {});
+            fp32_conv(c, rho, nullptr, c->d_vtab[cmp], c->d_psiv, st, [](int) {});
             usr::launch_grid_dot(c->grid, rho, c->d_psiv, 0.5, c->d_vpart, c->d_counters + 3, c->d_vdot + cmp, st);
         }
         usr::launch_virial_finalize(c->d_vnear, cluster_list(c), c->ncell, c->d_vdot, en, c->d_W, st);
@@ -999,7 +977,6 @@ usr_status init_ctx(usr_ctx* c, const usr_params* p)
         cudaGetLastError();
         return USR_ERR_CUDA;
     }
-    if ((s = usr::grid_kernel_setup(usr::kTileMaxSmem)) != USR_OK) return s;
     if ((s = usr::conv_tc_setup(false, usr::kConvTcMaxSmem)) != USR_OK ||
         (s = usr::conv_tc_setup(true, usr::kConvTcMaxSmem)) != USR_OK)
         return s;

@@ -38,6 +38,11 @@ constexpr int kCombineBlocks = 608;    // CTAs of the near + far combination at 
  * cell-list kernels before the fork trigger early: their successors' waiting CTAs then hold SM slots
  * nothing else needs, whereas waiting CTAs beside the pair kernel and the far chain slowed both.
  * Without the launch attribute (USR_PDL 0) both calls are no-ops and the launches are ordinary ones.
+ *
+ * Every kernel but the gather also asks for the largest shared-memory carve-out, though most need little of it:
+ * an SM changes its split between L1 and shared memory only when idle, and the far chain's convolutions, which
+ * need 100 KB and more, would otherwise wait until the pair kernel's persistent CTAs (or whatever else set a
+ * small carve-out) have left the SM.  carve < 0 leaves the choice to the driver (the gather lives on L1 hits).
  */
 #ifndef USR_PDL
 #define USR_PDL 1
@@ -47,19 +52,28 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+inline cudaError_t launch_with(int carve, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               A&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = USR_PDL;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = carve < 0 ? 0 : (unsigned int)carve;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = carve < 0 ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+{
+    return launch_with(cudaSharedmemCarveoutMaxShared, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 #endif
 #ifndef USR_GATHER_THREADS
@@ -71,27 +85,16 @@ inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t 
 constexpr int kGatherBlocks = USR_GATHER_BLOCKS;   // gather CTAs at most
 
 /*
- * Cell blocks of the spreading / interpolation kernels and their smem tiles.
- * Block b along axis a covers cells [b kb_a, min((b+1) kb_a, nc_a)); its tile
- * spans grid points org_a[b] .. org_a[b] + T_a - 1 (periodic).  The reduction
- * table lists, for every grid index g of axis a, the (block, tile offset)
- * pairs whose tile holds g: red_cnt_a[g] entries at red_pair_a[g * rmax_a].
+ * Blocks of cells and the grid tiles that hold the stencils of their atoms.  Block b along axis a covers
+ * cells [b kb_a, min((b+1) kb_a, nc_a)); its tile spans grid points org_a[b] .. org_a[b] + T_a - 1 (periodic).
+ * The plan's limit on cells (in grid points) is stated in these: a block of one cell must fit kTileMaxSmem.
  */
-constexpr int kTileMaxSmem = 112 * 1024;   // bytes per tile: two CTAs per SM
+constexpr int kTileMaxSmem = 112 * 1024;   // bytes per tile
 struct TileGeom {
     int kb[3];      // cells per block per axis
     int nbk[3];     // blocks per axis
     int T[3];       // tile extent per axis (grid points); T[0] % 4 == 0
-    int rmax[3];    // reduction-table row length per axis
-    int ps;         // plane stride of the tile in shared memory (floats, >= T[0] T[1], a multiple of 4), chosen
-                    // so that the spread's lanes hit distinct banks
-};
-
-/* Device copies of the per-axis tile tables (owned by the context). */
-struct TileTabs {
-    const int* org[3];
-    const int* red_cnt[3];
-    const int2* red_pair[3];
+    int ps;         // plane stride of the tile (floats, >= T[0] T[1], a multiple of 4)
 };
 
 /* Host plan: everything usr_init derives from usr_params, in FP64. */
@@ -135,8 +138,6 @@ struct Plan {
     int cells[3];
     TileGeom tile;
     std::vector<int> tile_org[3];        // per axis: tile origin of each block
-    std::vector<int> red_cnt[3];         // per axis: covering tiles of each grid index
-    std::vector<int> red_pair[3];        // per axis: (block, offset) pairs, rmax per grid index
 };
 
 /* Build the plan (host only).  Returns USR_OK or an error. */
@@ -170,9 +171,21 @@ struct BoxF {
     float invL[3];    // (float)(1/L)
     float cs[3];      // (float)(nc / L)
     float gs[3];      // (float)(n / L): grid coordinate scale
+    float gl[3];      // n / L - gs: what gs lacks of it
     int nc[3];
     int n[3];
 };
+
+#ifdef __CUDACC__
+/*
+ * Fractional grid coordinate of x on axis a, given cell = floor(x gs): x n / L - cell with one rounding of a number
+ * below 1 (x gs alone carries 2^-24 of a coordinate up to n, which the stencil weights amplify).
+ */
+__device__ __forceinline__ float grid_frac(const BoxF& b, int a, float x, float cell)
+{
+    return fmaf(x, b.gl[a], fmaf(x, b.gs[a], -cell));
+}
+#endif
 
 /*
  * Debug build (USR_DEBUG_BOUNDS defined): the kernels check their computed
@@ -236,8 +249,6 @@ struct GridArgs {
     float wsum;           // sum of the spreading weights over a stencil
     const double* psi_mean;   // grid mean of psi (its k = 0 mode, zero up to rounding)
     double F0d;           // the same in FP64 (self energy)
-    TileGeom tg;
-    TileTabs tab;
 };
 
 struct ConvGemm {
@@ -270,6 +281,7 @@ struct ConvTcArgs {
     int smem;               // dynamic shared memory per CTA (bytes; padded so that the CTAs an SM
                             // can hold never ask for more than 512 TMEM columns together)
     const float* mu;        // per-term mean of the 1D kernel (passes 1, 2)
+    const double* mean;     // pass 1: grid mean of A, taken off its row sums (may be null)
     void* out_hi;           // pass output (hi part; FP32 psi for pass 3)
     void* out_lo;           // pass output (lo part; unused for pass 3)
     int* status;
@@ -299,9 +311,9 @@ struct MlArgs {
 };
 
 // ---- launchers (all enqueue on `st`) ----
-/* rho (fine, [z][y][x]) -> rho_c (coarse) through t1 = [n2][n1][nc0], t2 = [n2][nc1][nc0]; with rho_c_lo
+/* rho less its grid mean (fine, [z][y][x]) -> rho_c (coarse) through t1 = [n2][n1][nc0], t2 = [n2][nc1][nc0]; with rho_c_lo
    non-null, rho_c / rho_c_lo receive the TF32 hi / lo split of the result (tensor-core coarse passes). */
-void launch_ml_restrict(const MlArgs& m, const float* rho, float* t1, float* t2, float* rho_c, float* rho_c_lo,
+void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c, float* rho_c_lo,
                         int* status, cudaStream_t st);
 /* psi += prolongation of psi_c, through t1 = [nc2][nc1][n0], t2 = [nc2][n1][n0] */
 void launch_ml_prolong(const MlArgs& m, const float* psi_c, float* t1, float* t2, float* psi, int* status,
@@ -330,9 +342,14 @@ void launch_near(int max_groups, int deg, const ClusterList& L, const NearArgs& 
 void set_near_ctas_per_sm(usr_ctx* c, int ctas_per_sm);
 void launch_pairs(int max_clusters, const ClusterList& L, const int* perm, const NearArgs& a, int* count,
                   unsigned long long* hash, int* status, cudaStream_t st);
-void launch_spread(int P, const float4* spos, const int* cell_start, const GridArgs& g, float* tilebuf, int split,
-                   void* rho, void* rho_lo, double* partial, unsigned int* counter, double* mean, int* status,
-                   cudaStream_t st, float* rho32 = nullptr);
+/* rho with its k = 0 mode still in it, as FP32 (split 0, rho) or a TF32 / BF16 operand split (1 / 2, rho and
+   rho_lo, and an FP32 copy in rho32 when that is non-null), and its grid mean through spread_ctas(n) partial sums */
+void launch_spread(int P, const float4* spos, const int* cell_start, const GridArgs& g, int split, void* rho,
+                   void* rho_lo, float* rho32, double* partial, unsigned int* counter, double* mean, int* status,
+                   cudaStream_t st);
+int spread_ctas(const int* n);
+/* out = rho - mean (in place when out is rho) */
+void launch_sub_mean(long long G, const float* rho, float* out, const double* mean, cudaStream_t st);
 void launch_grid_dot(const GridArgs& g, const float* a, const float* b, double scale, double* partial,
                      unsigned int* counter, double* out, cudaStream_t st);
 void launch_virial_finalize(const double* near_w, const ClusterList& L, int ncell, const double* dots,
@@ -357,8 +374,5 @@ void launch_combine(int n, const float4* spos, const int* perm, const unsigned l
                     const float4* far4, const GridArgs& g, float4* out, float4* near_dbg, float4* far_dbg,
                     double* partial, unsigned int* counter, double* energy, double* net_charge, int* status,
                     cudaStream_t st);
-int tile_blocks(const TileGeom& tg);
-size_t tile_floats(const TileGeom& tg);
-usr_status grid_kernel_setup(size_t smem_bytes);
 
 }  // namespace usr

@@ -465,25 +465,8 @@ usr_status make_plan(const usr_params* pp, Plan* out)
         for (int a = 0; a < 3; ++a) {
             const int H = P.P / 2;
             P.tile_org[a].resize(tg.nbk[a]);
-            std::vector<std::vector<int>> lists(P.n[a]);
-            for (int b = 0; b < tg.nbk[a]; ++b) {
-                const int o = (int)std::floor(b * tg.kb[a] * wg[a] + 1e-9) - H - 1;
-                P.tile_org[a][b] = o;
-                for (int t = 0; t < tg.T[a]; ++t) {
-                    const int gi = (((o + t) % P.n[a]) + P.n[a]) % P.n[a];
-                    lists[gi].push_back(b);
-                    lists[gi].push_back(t);
-                }
-            }
-            int rmax = 0;
-            for (auto& l : lists) rmax = std::max(rmax, (int)l.size() / 2);
-            tg.rmax[a] = rmax;
-            P.red_cnt[a].assign(P.n[a], 0);
-            P.red_pair[a].assign((size_t)P.n[a] * rmax * 2, 0);
-            for (int gi = 0; gi < P.n[a]; ++gi) {
-                P.red_cnt[a][gi] = (int)lists[gi].size() / 2;
-                std::copy(lists[gi].begin(), lists[gi].end(), P.red_pair[a].begin() + (size_t)gi * rmax * 2);
-            }
+            for (int b = 0; b < tg.nbk[a]; ++b)
+                P.tile_org[a][b] = (int)std::floor(b * tg.kb[a] * wg[a] + 1e-9) - H - 1;
         }
     }
     // the pair kernel evaluates F in FP32 (relative rounding ~6e-8): a fit error
