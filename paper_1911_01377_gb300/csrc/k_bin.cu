@@ -8,7 +8,8 @@
  *   place       scatter caller indices into their cell's range
  *   cell_sort   order each cell's atoms by caller index (a stable, run-to-run
  *               deterministic order) and gather the sorted float4 rows
- *   clusters    the pair kernel's 8-atom clusters, built from the sorted list
+ *   clusters    8-atom spatial clusters, the order every later kernel walks (an evaluation does not
+ *               run cell_sort)
  *
  * Predicate (per axis, RN rounding, no contraction):
  *   k = floorf(x * invL); xw = fmaf(-k, L, x); if (xw < 0) xw += L;
@@ -17,6 +18,8 @@
  * lengths) that the wrap leaves them outside [0, L], go to cell 0 at the
  * origin with charge 0 and raise the status word.
  */
+#include <climits>
+
 #include "usr_internal.h"
 
 namespace usr {
@@ -200,37 +203,25 @@ __global__ void __launch_bounds__(kSortThreads) k_cell_sort(int n, const int* __
 }
 
 /*
- * 8-atom clusters for the pair kernel, one CTA per cell: the cell's atoms
- * are ordered by the Morton code of their position on an 8 x 8 x 8 lattice
- * inside the cell (ties by sorted index), so that runs of 8 are compact;
- * written to the padded layout at pstart[c] with dummy rows (q = 0, far
- * away and far apart, index -1) after the last atom; then each cluster's
- * bounding box.
+ * 8-atom clusters for the pair kernel, one CTA per cell.  The cell's atoms are packed by sorting and
+ * tiling: sorted by x and cut into slabs, each slab sorted by y and cut into columns, each column sorted
+ * by z; every cut falls on a multiple of 8 atoms, so the clusters (runs of 8) are disjoint boxes of about
+ * equal edges.  About cbrt(clusters) slabs and the square root of a slab's clusters as columns.  Written to
+ * the padded layout at pstart[c] as (x, y, z, q) rows with dummy rows (q = 0, far away and far apart, index
+ * -1) after the last atom; then each cluster's bounding box.
  *
- * Cluster positions are stored paired for the pair kernel's two-wide FP32
- * arithmetic: atom t of a cluster (t = 4 h + g, h = 0, 1) goes to the 32-byte
- * group g as x at float 8 g + h, y at 8 g + 2 + h, z at 8 g + 4 + h and q at
- * 8 g + 6 + h, so one lane's two 16-byte loads give (x_g, x_g+4), (y_g, y_g+4),
- * (z_g, z_g+4), (q_g, q_g+4).
+ * The pair kernel's work is the 8 x 8 cluster pairs whose boxes come within r_c.  Against runs of 8 along a
+ * Morton curve on an 8 x 8 x 8 lattice in the cell (the earlier order, whose runs straddle octants) tiling
+ * leaves 20 % fewer of them on the slab at r_c = 10 A and 23 % fewer on water at r_c = 9 A (counted on the
+ * CPU), the same as recursive median splits, for three rank-by-counting passes of which the second and third
+ * only run over a slab and a column.  The Morton order remains for cells of more than kTileMax atoms, whose
+ * three keys do not fit the shared arrays (densities far above the method's).
  */
+constexpr int kTileMax = 1024;
+
 __device__ __forceinline__ int spread3(int v)
 {
     return (v & 1) | ((v & 2) << 2) | ((v & 4) << 4);
-}
-
-__device__ __forceinline__ int pk_off(int slot)
-{
-    const int t = slot & 7;
-    return (slot >> 3) * 32 + 8 * (t & 3) + (t >> 2);
-}
-
-__device__ __forceinline__ void pk_store(float* cp, int slot, float4 p)
-{
-    const int o = pk_off(slot);
-    cp[o] = p.x;
-    cp[o + 2] = p.y;
-    cp[o + 4] = p.z;
-    cp[o + 6] = p.w;
 }
 
 __device__ __forceinline__ int morton_key(float4 p, float ox, float oy, float oz, float kx, float ky, float kz)
@@ -241,93 +232,166 @@ __device__ __forceinline__ int morton_key(float4 p, float ox, float oy, float oz
     return spread3(ix) | (spread3(iy) << 1) | (spread3(iz) << 2);
 }
 
+/* Sorting key of a coordinate u (from the cell's corner): its float bits, then the caller index, so that keys are
+   distinct and their order does not depend on the order in which the cell's entries were placed. */
+__device__ __forceinline__ long long tile_key(float u, int x)
+{
+    return ((long long)__float_as_int(fmaxf(u, 0.f)) << 32) | (unsigned int)x;
+}
+
+/* How many of k[lo .. hi) are below ke; lo is a multiple of 8 and k is padded with LLONG_MAX to hi. */
+__device__ __forceinline__ int rank_of(const long long* k, int lo, int hi, long long ke)
+{
+    int r = 0;
+    #pragma unroll 2
+    for (int f = lo; f < hi; f += 4) {
+        const longlong2 v = *reinterpret_cast<const longlong2*>(k + f);
+        const longlong2 w = *reinterpret_cast<const longlong2*>(k + f + 2);
+        r += v.x < ke;
+        r += v.y < ke;
+        r += w.x < ke;
+        r += w.y < ke;
+    }
+    return r;
+}
+
 /*
- * The clusters of one cell per CTA, from the sorted cell list (k_cell_sort):
- * Morton order as above, the padded paired layout, each cluster's bounding
- * box; also the first cluster of each of the cell's groups of gcl clusters,
- * and the cell's rows of the pair kernel's fixed-point accumulators set to
- * zero.  A separate kernel from the sort, so that the far part, which needs
- * only the sorted list, can start beside it on another stream.
+ * The clusters of one cell per CTA, from the cell's entries in any order (k_place): the packing above, the padded
+ * layout, each cluster's bounding box; also the descriptor of each of the cell's groups of gcl clusters, and the
+ * cell's rows of the pair kernel's fixed-point accumulators (four per slot) set to zero.  The pair kernel, the
+ * spreading, the gather and the combination all walk the slots, so an evaluation needs no other order of the atoms.
  */
-__global__ void __launch_bounds__(kSortThreads) k_cluster_build(const int* __restrict__ start,
-                                                                const int* __restrict__ pstart,
-                                                                const int* __restrict__ gfull,
-                                                                const int* __restrict__ gpart, int gcl, BoxF b,
-                                                                const float4* __restrict__ spos,
-                                                                int* __restrict__ key, float4* __restrict__ cpos,
-                                                                int* __restrict__ cidx, int* __restrict__ ccell,
-                                                                float4* __restrict__ bblo, float4* __restrict__ bbhi,
-                                                                int* __restrict__ gfirst,
-                                                                unsigned long long* __restrict__ acc, int n,
-                                                                int max_slots, int max_groups,
-                                                                int* __restrict__ status)
+__global__ void __launch_bounds__(256) k_cluster_build(const int* __restrict__ start,
+                                                       const int* __restrict__ pstart,
+                                                       const int* __restrict__ gfull,
+                                                       const int* __restrict__ gpart, int gcl, BoxF b,
+                                                       const int* __restrict__ unsorted,
+                                                       const float4* __restrict__ wpos,
+                                                       int* __restrict__ key, float4* __restrict__ cpos,
+                                                       int* __restrict__ cperm, int* __restrict__ ccell,
+                                                       float4* __restrict__ bblo, float4* __restrict__ bbhi,
+                                                       int4* __restrict__ gdesc,
+                                                       unsigned long long* __restrict__ acc, int n,
+                                                       int max_slots, int max_groups, int* __restrict__ status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
-    __shared__ int ks[kSortMax];
+    __shared__ __align__(16) long long k0[kTileMax], k1[kTileMax];
+    const int threads = blockDim.x;
     const int c = blockIdx.x;
     const int s0 = start[c], m = start[c + 1] - s0;
     const int p0 = pstart[c], pm = pstart[c + 1] - p0;
     if (pm == 0) return;                                  // an empty cell has no clusters
-    const int cx = c % b.nc[0], cy = (c / b.nc[0]) % b.nc[1], cz = c / (b.nc[0] * b.nc[1]);
-    const float ox = (float)cx / b.cs[0], oy = (float)cy / b.cs[1], oz = (float)cz / b.cs[2];
-    const float kx = 8.0f * b.cs[0], ky = 8.0f * b.cs[1], kz = 8.0f * b.cs[2];
-    const bool in_smem = m <= kSortMax;
-    float* cp = reinterpret_cast<float*>(cpos);
+    if (!USR_IN_BOUNDS(s0 + m - 1, n, status) || !USR_IN_BOUNDS(p0 + pm - 1, max_slots, status)) return;
     {
         // full groups in cell order, then the partial ones (the pair kernel takes them in that order,
         // so its last work units are the small ones)
         const int f0 = gfull[c], nf = gfull[c + 1] - f0;
-        for (int k = threadIdx.x; k < nf; k += kSortThreads)
-            if (USR_IN_BOUNDS(f0 + k, max_groups, status)) gfirst[f0 + k] = (p0 >> 3) + k * gcl;
+        for (int k = threadIdx.x; k < nf; k += threads)
+            if (USR_IN_BOUNDS(f0 + k, max_groups, status)) gdesc[f0 + k] = make_int4((p0 >> 3) + k * gcl, c, gcl, 0);
         if (threadIdx.x == 0 && gpart[c + 1] > gpart[c]) {
             const int gp = gfull[b.nc[0] * b.nc[1] * b.nc[2]] + gpart[c];
-            if (USR_IN_BOUNDS(gp, max_groups, status)) gfirst[gp] = (p0 >> 3) + nf * gcl;
+            if (USR_IN_BOUNDS(gp, max_groups, status))
+                gdesc[gp] = make_int4((p0 >> 3) + nf * gcl, c, (pm >> 3) - nf * gcl, 0);
         }
-        if (USR_IN_BOUNDS(s0 + m - 1, n, status)) {
-            ulonglong2* a2 = reinterpret_cast<ulonglong2*>(acc + 4 * (size_t)s0);
-            for (int e = threadIdx.x; e < 2 * m; e += kSortThreads) a2[e] = make_ulonglong2(0ull, 0ull);
+        ulonglong2* a2 = reinterpret_cast<ulonglong2*>(acc + 4 * (size_t)p0);
+        for (int e = threadIdx.x; e < 2 * pm; e += threads) a2[e] = make_ulonglong2(0ull, 0ull);
+    }
+    const int cx = c % b.nc[0], cy = (c / b.nc[0]) % b.nc[1], cz = c / (b.nc[0] * b.nc[1]);
+    const float ox = (float)cx / b.cs[0], oy = (float)cy / b.cs[1], oz = (float)cz / b.cs[2];
+    if (m <= kTileMax) {
+        const int ncl = pm >> 3;
+        int sx = 1;                                       // slabs: the cube root of the clusters, rounded
+        while ((2 * sx + 1) * (2 * sx + 1) * (2 * sx + 1) <= 8 * ncl) ++sx;
+        for (int e = threadIdx.x; e < pm; e += threads) {
+            const int x = e < m ? unsorted[s0 + e] : 0;
+            k0[e] = e < m ? tile_key(wpos[x].x - ox, x) : LLONG_MAX;
+        }
+        __syncthreads();
+        // each pass puts every atom at its place in the next order and stores its next key there
+        for (int e = threadIdx.x; e < pm; e += threads) {
+            if (e < m) {
+                const long long ke = k0[e];
+                const int r = rank_of(k0, 0, pm, ke), x = (int)ke;
+                k1[r] = tile_key(wpos[x].y - oy, x);
+            } else {
+                k1[e] = LLONG_MAX;
+            }
+        }
+        __syncthreads();
+        // slab s holds the clusters [ncl s / sx, ncl (s + 1) / sx); column y of its kc clusters likewise
+        for (int r = threadIdx.x; r < pm; r += threads) {
+            const int s = (((r >> 3) + 1) * sx - 1) / ncl;
+            const int a0 = 8 * (ncl * s / sx), a1 = 8 * (ncl * (s + 1) / sx);
+            if (r < m) {
+                const long long kr = k1[r];
+                const int x = (int)kr;
+                k0[a0 + rank_of(k1, a0, a1, kr)] = tile_key(wpos[x].z - oz, x);
+            } else {
+                k0[r] = LLONG_MAX;
+            }
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < m; q += threads) {
+            const int s = (((q >> 3) + 1) * sx - 1) / ncl;
+            const int l0 = ncl * s / sx, kc = ncl * (s + 1) / sx - l0;
+            int sy = 1;                                   // columns: the square root of the slab's clusters, rounded
+            while ((2 * sy + 1) * (2 * sy + 1) <= 4 * kc) ++sy;
+            const int y = (((q >> 3) - l0 + 1) * sy - 1) / kc;
+            const int b0 = 8 * (l0 + kc * y / sy), b1 = 8 * (l0 + kc * (y + 1) / sy);
+            const long long kq = k0[q];
+            const int t = b0 + rank_of(k0, b0, b1, kq), x = (int)kq;
+            cpos[p0 + t] = wpos[x];
+            cperm[p0 + t] = x;
+        }
+    } else {
+        const float fx = 8.0f * b.cs[0], fy = 8.0f * b.cs[1], fz = 8.0f * b.cs[2];
+        int* kk = key + s0;
+        const int* xs = unsorted + s0;
+        for (int e = threadIdx.x; e < m; e += threads) kk[e] = morton_key(wpos[xs[e]], ox, oy, oz, fx, fy, fz);
+        __syncthreads();
+        for (int e = threadIdx.x; e < m; e += threads) {
+            const int ke = kk[e], x = xs[e];
+            int r = 0;
+            for (int f = 0; f < m; ++f) {
+                const int kf = kk[f];
+                r += (kf < ke) || (kf == ke && xs[f] < x);
+            }
+            cpos[p0 + r] = wpos[x];
+            cperm[p0 + r] = x;
         }
     }
-    int* kk = in_smem ? ks : key + s0;
-    if (!USR_IN_BOUNDS(s0 + m - 1, n, status)) return;
-    // cluster order: Morton code of each atom on an 8 x 8 x 8 lattice inside the cell, ties by sorted index
-    for (int e = threadIdx.x; e < m; e += kSortThreads) kk[e] = morton_key(spos[s0 + e], ox, oy, oz, kx, ky, kz);
-    __syncthreads();
-    for (int e = threadIdx.x; e < m; e += kSortThreads) {
-        const int ke = kk[e];
-        int r = 0;
-        for (int f = 0; f < m; ++f) {
-            const int kf = kk[f];
-            r += (kf < ke) || (kf == ke && f < e);
-        }
-        if (!USR_IN_BOUNDS(p0 + r, max_slots, status)) continue;
-        pk_store(cp, p0 + r, spos[s0 + e]);
-        cidx[p0 + r] = s0 + e;
-    }
-    for (int e = m + threadIdx.x; e < pm; e += kSortThreads) {
-        if (!USR_IN_BOUNDS(p0 + e, max_slots, status)) continue;
+    for (int e = m + threadIdx.x; e < pm; e += threads) {
         // padding rows: far from the box, so never within r_c of an atom, and 4e4 A apart within
         // a cluster (rows of different cells may coincide; the pair kernel never uses their sums)
         const float far = -1.0e6f - 4.0e4f * (float)(e & 7);
-        pk_store(cp, p0 + e, make_float4(far, far, far, 0.0f));
-        cidx[p0 + e] = -1;
+        cpos[p0 + e] = make_float4(far, far, far, 0.0f);
+        cperm[p0 + e] = -1;
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < (pm >> 3); k += kSortThreads) {
+    // bounding boxes: eight lanes per cluster (pm is a multiple of 8, so a cluster's lanes run together)
+    for (int e = threadIdx.x; e < pm; e += threads) {
         float4 lo = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f), hi = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
-        for (int t = 0; t < 8; ++t) {
-            const int sl = p0 + 8 * k + t;
-            if (cidx[sl] < 0) continue;
-            const int o = pk_off(sl);
-            const float4 p = make_float4(cp[o], cp[o + 2], cp[o + 4], 0.f);
-            lo.x = fminf(lo.x, p.x); lo.y = fminf(lo.y, p.y); lo.z = fminf(lo.z, p.z);
-            hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
+        if (e < m) {
+            const float4 p = cpos[p0 + e];
+            lo = make_float4(p.x, p.y, p.z, 0.f);
+            hi = lo;
         }
-        const int cl = (p0 >> 3) + k;
-        if (!USR_IN_BOUNDS(cl, max_slots >> 3, status)) continue;
-        bblo[cl] = lo;
-        bbhi[cl] = hi;
-        ccell[cl] = c;
+        const unsigned int peers = 0xffu << (threadIdx.x & 24);
+        #pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            lo.x = fminf(lo.x, __shfl_xor_sync(peers, lo.x, o));
+            lo.y = fminf(lo.y, __shfl_xor_sync(peers, lo.y, o));
+            lo.z = fminf(lo.z, __shfl_xor_sync(peers, lo.z, o));
+            hi.x = fmaxf(hi.x, __shfl_xor_sync(peers, hi.x, o));
+            hi.y = fmaxf(hi.y, __shfl_xor_sync(peers, hi.y, o));
+            hi.z = fmaxf(hi.z, __shfl_xor_sync(peers, hi.z, o));
+        }
+        if ((e & 7) == 0) {
+            const int cl = (p0 + e) >> 3;
+            bblo[cl] = lo;
+            bbhi[cl] = hi;
+            ccell[cl] = c;
+        }
     }
 }
 
@@ -348,10 +412,10 @@ cudaError_t launch_bin(int n, const float4* xyzq, const BoxF& b, int ncell, int*
     return cudaGetLastError();
 }
 
-/* The sorted cell list: counts, scan (with the pair kernel's group counts), placement, per-cell sort. */
-void launch_bin_sorted(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
-                       float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue, int* unsorted,
-                       int* perm, float4* spos, int* status, cudaStream_t st)
+/* The cell list: counts, scan (with the pair kernel's group counts), placement (any order within a cell). */
+void launch_bin_list(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
+                     float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue, int* unsorted,
+                     int* status, cudaStream_t st)
 {
     // count[] is zero on entry: the context zeroes it when it is (re)configured, and k_scan zeroes every
     // entry after reading it, ready for the next evaluation (no memset between the kernels)
@@ -360,17 +424,25 @@ void launch_bin_sorted(int n, const float4* xyzq, const BoxF& b, int ncell, int*
     launch_pdl(k_bin_count, nb, 256, 0, st, n, xyzq, b, count, cell_of, slot, wpos, status);
     launch_pdl(k_scan, 1, 1024, 0, st, ncell, count, cell_start, pstart, gfull, gpart, gcl, queue);
     launch_pdl(k_place, nb, 256, 0, st, n, cell_of, slot, cell_start, unsorted, status);
+}
+
+/* Each cell's atoms in the order of their caller indices (the canonical order of the inspection entry points). */
+void launch_cell_sort(int n, int ncell, const int* cell_start, const int* unsorted, const float4* wpos, int* perm,
+                      float4* spos, int* status, cudaStream_t st)
+{
     launch_pdl(k_cell_sort, ncell, kSortThreads, 0, st, n, cell_start, unsorted, wpos, perm, spos, status);
 }
 
-/* The pair kernels' clusters from the sorted cell list (slot[] of launch_bin_sorted is reused for keys). */
+/* The clusters from the cell list (slot[] of launch_bin_list is reused for keys). */
 void launch_clusters(int n, const BoxF& b, int ncell, const int* cell_start, const int* pstart, const int* gfull,
-                     const int* gpart, int* gfirst, const float4* spos, int* key, float4* cpos, int* cidx,
-                     int* ccell, float4* bblo, float4* bbhi, unsigned long long* near_acc, int max_clusters,
-                     int max_groups, int* status, cudaStream_t st)
+                     const int* gpart, int4* gdesc, const int* unsorted, const float4* wpos, int* key, float4* cpos,
+                     int* cperm, int* ccell, float4* bblo, float4* bbhi, unsigned long long* near_acc,
+                     int max_clusters, int max_groups, int* status, cudaStream_t st)
 {
-    launch_pdl(k_cluster_build, ncell, kSortThreads, 0, st, cell_start, pstart, gfull, gpart, near_group_clusters(),
-               b, spos, key, cpos, cidx, ccell, bblo, bbhi, gfirst, near_acc, n, 8 * max_clusters, max_groups,
+    // a thread per atom of a mean cell, within 128 and 256
+    const int threads = n > 128LL * ncell ? 256 : 128;
+    launch_pdl(k_cluster_build, ncell, threads, 0, st, cell_start, pstart, gfull, gpart, near_group_clusters(), b,
+               unsorted, wpos, key, cpos, cperm, ccell, bblo, bbhi, gdesc, near_acc, n, 8 * max_clusters, max_groups,
                status);
 }
 

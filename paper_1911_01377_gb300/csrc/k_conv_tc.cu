@@ -24,9 +24,9 @@
  * Precision: operands are split into high and low parts, A = A_hi + A_lo,
  * B = B_hi + B_lo, and D = A_hi B_hi + A_hi B_lo + A_lo B_hi is accumulated in
  * FP32 (three MMAs per k-step): TF32x3 (10 + 10 mantissa bits per operand)
- * or BF16x3 (7 + 8).  The tensor core truncates each addition to its FP32 sum, so the two small products
- * have an accumulator of their own (NT further columns), which saves the large one two truncations of three;
- * the epilogue adds the two.  Each epilogue writes the hi and lo parts of its output
+ * or BF16x3 (7 + 8).  The tensor core truncates each addition to its FP32 sum, so in the TF32 form
+ * the two small products have an accumulator of their own (NT further columns), which saves the large one two
+ * truncations of three; the epilogue adds the two (BF16x3's operand rounding is larger than that).  Each epilogue writes the hi and lo parts of its output
  * for the next pass; the last writes FP32.
  *
  * CTA: 128 threads, one 128-line M tile, one N tile of NT <= 256 columns
@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_sh;
+    const uint32_t small = BF16 ? 0u : (uint32_t)NT;   // columns of the small products' sums
 
     const int a_row = batch * g.a_rows_per_batch + m0;
     const int b_row = (batch * g.ntiles + tile) * NT;
@@ -284,8 +285,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
                 const uint64_t off = (uint64_t)((k * KMMA * (BF16 ? 2 : 4)) >> 4);   // bytes along the row
                 const uint32_t first = (kb == 0 && k == 0) ? 0u : 1u;
                 mma<BF16>(tmem, ah + off, bh + off, idesc, first);
-                mma<BF16>(tmem + NT, ah + off, bl + off, idesc, first);
-                mma<BF16>(tmem + NT, al + off, bh + off, idesc, 1u);
+                mma<BF16>(tmem + small, ah + off, bl + off, idesc, BF16 ? 1u : first);
+                mma<BF16>(tmem + small, al + off, bh + off, idesc, 1u);
             }
             mma_commit(empty0 + 8 * s);            // the stage is free once these MMAs have read it
         }
@@ -310,11 +311,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
         // the DC column sits right after the tile's real columns
         const int dcc = g.cols;
         tmem_ld16(trow + (uint32_t)(dcc & ~15), v);
-        tmem_ld16(trow + (uint32_t)(NT + (dcc & ~15)), w);
+        if (!BF16) tmem_ld16(trow + small + (uint32_t)(dcc & ~15), w);
         float dc = 0.f;
         #pragma unroll
         for (int i = 0; i < 16; ++i)
-            if (i == (dcc & 15)) dc = v[i] + w[i];
+            if (i == (dcc & 15)) dc = BF16 ? v[i] : v[i] + w[i];
         const bool valid = line < g.lines;
         const int c_lo = tile * g.cols;
         float muj = 0.f;
@@ -328,11 +329,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
         }
         for (int c0 = 0; c0 < g.cols; c0 += 16) {
             tmem_ld16(trow + (uint32_t)c0, v);
-            tmem_ld16(trow + (uint32_t)(NT + c0), w);
+            if (!BF16) tmem_ld16(trow + small + (uint32_t)c0, w);
             if (!valid) continue;
             #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                v[i] += w[i];
+                if (!BF16) v[i] += w[i];
                 const int c = c0 + i;
                 const int m = c_lo + c;
                 if (c >= g.cols || m >= g.n_out) continue;

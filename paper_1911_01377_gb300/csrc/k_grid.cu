@@ -4,13 +4,16 @@
  * combination with the near part, atomic-free and deterministic.
  *
  *   gather   phi_far,i = sum_g w(g - r_i) psi_g and F_far,i = -q_i grad phi_far,i
- *            (the second spreading Gaussian of Eq. 32's 1/|S(k)|^2), per sorted
- *            atom, reading psi from global memory; contracts the stencil
+ *            (the second spreading Gaussian of Eq. 32's 1/|S(k)|^2), per cluster
+ *            slot, reading psi from global memory; contracts the stencil
  *            separably (z first, per (x, y) column); also psi's grid mean.
  *   combine  after the pair kernel: near + far + the self term -F(0) q_i in
  *            caller order, and E = 1/2 sum q_i phi_i and its parts
  *            (compensated FP32 within a warp, FP64 across warps and blocks).
  */
+#include <algorithm>
+#include <climits>
+
 #include "usr_internal.h"
 
 namespace usr {
@@ -165,20 +168,20 @@ void launch_virial_finalize(const double* near_w, const ClusterList& L, int ncel
 
 /* ------------------------------------------------------------------ gather */
 
-/* The pair kernel's near part of sorted atom s: four fixed-point sums (2^-32 units) as FP32. */
-__device__ __forceinline__ float4 near_part(const unsigned long long* __restrict__ acc, int s)
+/* The pair kernel's near part of a cluster slot: four fixed-point sums (2^-32 units; component c of slot t of a
+   cluster at 8 c + t) as FP32. */
+__device__ __forceinline__ float4 near_part(const unsigned long long* __restrict__ acc, int slot)
 {
-    const ulonglong2* a2 = reinterpret_cast<const ulonglong2*>(acc + 4 * (size_t)s);
-    const ulonglong2 u = a2[0], v = a2[1];
+    const unsigned long long* a = acc + 32 * (size_t)(slot >> 3) + (slot & 7);
     constexpr float k = 2.3283064365386963e-10f;   // 2^-32, exact
-    return make_float4(__ll2float_rn((long long)u.x) * k, __ll2float_rn((long long)u.y) * k,
-                       __ll2float_rn((long long)v.x) * k, __ll2float_rn((long long)v.y) * k);
+    return make_float4(__ll2float_rn((long long)a[0]) * k, __ll2float_rn((long long)a[8]) * k,
+                       __ll2float_rn((long long)a[16]) * k, __ll2float_rn((long long)a[24]) * k);
 }
 
 /*
- * Far part at every sorted atom (the gather of Sec. V: the spreading Gaussian of the atom against psi,
- * and its gradient), read straight from psi in global memory: consecutive sorted atoms are neighbours in
- * space, so a CTA's stencils overlap and hit in L1 / L2.  A CTA takes consecutive atoms, gather_lanes(P)
+ * Far part at every cluster slot (the gather of Sec. V: the spreading Gaussian of the atom against psi,
+ * and its gradient), read straight from psi in global memory: consecutive slots are neighbours in
+ * space, so a CTA's stencils overlap and hit in L1 / L2.  A CTA takes consecutive slots, gather_lanes(P)
  * lanes per atom: lane u takes the stencil columns x = u, u + lanes, ... of every row, contracting z first,
  * so the lanes of an atom read one contiguous run of a row per load.  Writes far4[s] = (-q grad phi, phi
  * before the k = 0 correction); the CTAs also sum psi, and the last one writes its mean.
@@ -198,7 +201,7 @@ __host__ __device__ constexpr int gather_lanes(int P)
 
 template <int P>
 __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 256 / kGThreads)
-    k_gather(const float4* __restrict__ pos, int n, const float* __restrict__ psi, GridArgs g,
+    k_gather(const float4* __restrict__ cpos, const int* __restrict__ nslots, const float* __restrict__ psi, GridArgs g,
              float4* __restrict__ far4, double* __restrict__ partial, unsigned int* __restrict__ counter,
              double* __restrict__ psi_mean, int* __restrict__ status)
 {
@@ -219,10 +222,13 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
     const long long G = plane * n2;
     for (long long i = (long long)blockIdx.x * kGThreads + threadIdx.x; i < G; i += (long long)gridDim.x * kGThreads)
         ps.add(psi[i]);
-    for (int s0 = blockIdx.x * APC + warp * APW; s0 < n; s0 += gridDim.x * APC) {
+    const int ns = *nslots;
+    for (int s0 = blockIdx.x * APC + warp * APW; s0 < ns; s0 += gridDim.x * APC) {
         const int s = s0 + slot;
-        const bool have = slot < APW && s < n;     // lanes past APW x LPA hold no atom
-        const float4 p = pos[have ? s : s0];
+        // lanes past APW x LPA hold no atom, and neither do the padding slots (near -1e6)
+        float4 p = slot < APW && s < ns ? cpos[s] : make_float4(-1.0e6f, 0.f, 0.f, 0.f);
+        const bool have = p.x > -5.0e5f;
+        if (!have) p = make_float4(0.f, 0.f, 0.f, 0.f);
         const float pc[3] = {p.x, p.y, p.z};
         int base[3];
         float tt[3];
@@ -303,7 +309,7 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
                 az += __shfl_down_sync(0xffffffffu, p3, o);
             }
         }
-        if (have && u == 0 && USR_IN_BOUNDS(s, g.max_atoms, status)) {
+        if (have && u == 0 && USR_IN_BOUNDS(s, g.max_slots, status)) {
             const float qi = p.w;
             far4[s] = make_float4(-qi * ax, -qi * ay, -qi * az, aphi);
         }
@@ -337,15 +343,16 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
 }
 
 /*
- * After the pair kernel and the far gather: per sorted atom s, the result in caller order,
- *   out[perm[s]] = (F_near + F_far, phi_near + phi_far - F(0) q),
+ * After the pair kernel and the far gather: per cluster slot t that holds an atom, the result in caller order,
+ *   out[cperm[t]] = (F_near + F_far, phi_near + phi_far - F(0) q),
  * and the energies E = E_near + E_far + E_self (1/2 sum q phi over Eq. 20's near part, over the grid part,
  * and the self term -1/2 F(0) sum q^2), plus the net charge sum q (a diagnostic: the k = 0 term that a
  * non-zero net charge would carry is the one Eq. 4 drops).  Each block forms the four sums of its atoms;
  * the last block reduces them in block order.
  */
-__global__ void __launch_bounds__(kThreads) k_combine(int n, const float4* __restrict__ pos,
-                                                      const int* __restrict__ perm,
+__global__ void __launch_bounds__(kThreads) k_combine(const float4* __restrict__ cpos,
+                                                      const int* __restrict__ cperm,
+                                                      const int* __restrict__ nslots,
                                                       const unsigned long long* __restrict__ near_acc,
                                                       const float4* __restrict__ far4, float F0, double F0d,
                                                       float wsum, const double* __restrict__ psi_mean,
@@ -362,11 +369,13 @@ __global__ void __launch_bounds__(kThreads) k_combine(int n, const float4* __res
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float phi_dc = (float)(*psi_mean) * wsum;   // potential of psi's rounding-level k = 0 mode
     CSum qn, qf, qq, qs;                              // sums of q phi_near, q phi_far, q^2, q
-    for (int s = blockIdx.x * kThreads + threadIdx.x; s < n; s += gridDim.x * kThreads) {
-        const float4 nr = near_part(near_acc, s), f = far4[s];
-        const float qi = pos[s].w;
+    const int ns = *nslots;
+    for (int t = blockIdx.x * kThreads + threadIdx.x; t < ns; t += gridDim.x * kThreads) {
+        const int i = cperm[t];
+        const float4 nr = near_part(near_acc, t), f = far4[t];
+        const float qi = cpos[t].w;
+        if (i < 0) continue;                          // a padding slot
         const float phi_far = f.w - phi_dc;
-        const int i = perm[s];
         qn.add_product(qi, nr.w);
         qf.add_product(qi, phi_far);
         qq.add_product(qi, qi);
@@ -417,8 +426,11 @@ __global__ void __launch_bounds__(kThreads) k_combine(int n, const float4* __res
 
 #define USR_GATHER_CASE(PP)                                                                \
     case PP:                                                                               \
-        launch_with(-1, k_gather<PP>, nb, kGThreads, 0, st, spos, n, psi, g, far4, partial, counter, psi_mean, status); \
+        launch_with(-1, k_gather<PP>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, psi, g, far4, partial, counter, psi_mean, status); \
         break;
+
+/* Cluster slots of n atoms in ncell cells at most. */
+static int max_slots_of(int n, int ncell) { return (int)std::min((long long)n + 7LL * std::min(n, ncell), (long long)INT_MAX); }
 
 static int gather_blocks(int n, int P)
 {
@@ -426,10 +438,10 @@ static int gather_blocks(int n, int P)
     return std::max(1, std::min(kGatherBlocks, (n + apc - 1) / apc));
 }
 
-void launch_gather(int P, int n, const float4* spos, const float* psi, const GridArgs& g, float4* far4,
+void launch_gather(int P, int n, const ClusterList& L, int ncell, const float* psi, const GridArgs& g, float4* far4,
                    double* partial, unsigned int* counter, double* psi_mean, int* status, cudaStream_t st)
 {
-    const int nb = gather_blocks(n, P);
+    const int nb = gather_blocks(max_slots_of(n, ncell), P);
     switch (P) {
         USR_GATHER_CASE(8)
         USR_GATHER_CASE(10)
@@ -440,14 +452,13 @@ void launch_gather(int P, int n, const float4* spos, const float* psi, const Gri
     }
 }
 
-void launch_combine(int n, const float4* spos, const int* perm, const unsigned long long* near_acc,
-                    const float4* far4, const GridArgs& g, float4* out,
-                    float4* near_dbg, float4* far_dbg, double* partial, unsigned int* counter, double* energy,
-                    double* net_charge, int* status, cudaStream_t st)
+void launch_combine(int n, const ClusterList& L, int ncell, const unsigned long long* near_acc, const float4* far4,
+                    const GridArgs& g, float4* out, float4* near_dbg, float4* far_dbg, double* partial,
+                    unsigned int* counter, double* energy, double* net_charge, int* status, cudaStream_t st)
 {
-    const int nb = std::max(1, std::min(kCombineBlocks, (n + kThreads - 1) / kThreads));
-    k_combine<<<nb, kThreads, 0, st>>>(n, spos, perm, near_acc, far4, g.F0, g.F0d, g.wsum, g.psi_mean, out,
-                                       near_dbg, far_dbg, partial, counter, energy, net_charge, g.max_atoms,
+    const int nb = std::max(1, std::min(kCombineBlocks, (max_slots_of(n, ncell) + kThreads - 1) / kThreads));
+    k_combine<<<nb, kThreads, 0, st>>>(L.cpos, L.cperm, L.pstart + ncell, near_acc, far4, g.F0, g.F0d, g.wsum,
+                                       g.psi_mean, out, near_dbg, far_dbg, partial, counter, energy, net_charge, n,
                                        status);
 }
 

@@ -47,9 +47,6 @@
 #define USR_NEAR_MINB 5     // CTAs of 128 threads per SM the register budget is set for (96 registers:
                             // 20 warps per SM, 122 us at r_c = 10 A on the slab against 133 us with 16)
 #endif
-#ifndef USR_NEAR_NEWTON
-#define USR_NEAR_NEWTON 0
-#endif
 
 namespace usr {
 
@@ -96,88 +93,81 @@ __device__ __forceinline__ float exp2_ftz(float x)
 constexpr float kFixScale = 4294967296.0f;   // 2^32 fixed-point units per unit of force or potential
 constexpr float kFixMax = 1073741824.0f;     // 2^30: largest magnitude one part may carry
 
-/* Add v to a fixed-point accumulator (nothing for 0; status bit 8 for a part out of range or NaN). */
+/* Add v to a fixed-point accumulator (status bit 8 for a part out of range or NaN). */
 __device__ __forceinline__ void red_fix(unsigned long long* p, float v, int* status)
 {
     if (!(fabsf(v) < kFixMax)) {
         atomicOr(status, 8);
         return;
     }
-    const long long q = __float2ll_rn(v * kFixScale);
-    if (q != 0) atomicAdd(p, (unsigned long long)q);   // two's complement: a signed add
+    atomicAdd(p, (unsigned long long)__float2ll_rn(v * kFixScale));   // two's complement: a signed add
 }
-
-/* One i-cluster of the group, seen by a lane: atoms gi and gi + 4 and their sums. */
-struct NearI {
-    f2 x, y, z, q;
-    f2 fx, fy, fz, ph;
-};
 
 struct NearVir {
     f2 xx, yy, zz, xy, xz, yz;
 };
 
+/* i-side sums of one i-cluster, seen by a lane: atoms gi and gi + 4. */
+struct NearSum {
+    f2 x, y, z, p;
+};
+
 /*
- * One 8 x 8 step between i-cluster I and the lane's j atom (xj/yj/zj: minus its
- * position shifted to the image, duplicated into both halves).  Padding rows
- * never pass the distance test: as j atoms they sit near -1e6 (cpos), as i atoms
- * near +1e7 (replaced when the group is loaded).  TRI: the j-cluster is I
- * itself, only pairs with j after i count (tri_a / tri_b for halves a / b).
+ * One 8 x 8 step between the i atoms in A = (x, x', y, y'), B = (z, z', q, q') (atoms gi and gi + 4 of an
+ * i-cluster) and the lane's j atom (xj/yj/zj: minus its position shifted to the image, duplicated into both
+ * halves).  Padding rows never pass the distance test: as j atoms they sit near -1e6 (cpos), as i atoms near
+ * +1e7 (replaced when the group is loaded).  TRI: the j-cluster is the i-cluster itself, only pairs with j
+ * after i count (tri_a / tri_b for halves a / b).
  */
 template <int DEG, int NEXP, bool VIR, bool TRI>
-__device__ __forceinline__ void pair_step(const NearArgs& a, NearI& I, f2 xj, f2 yj, f2 zj, float qj, bool tri_a,
-                                          bool tri_b, f2& fjx, f2& fjy, f2& fjz, f2& fjp, NearVir& V)
+__device__ __forceinline__ void pair_step(const NearArgs& a, float4 A, float4 B, NearSum& I, f2 xj, f2 yj, f2 zj,
+                                          float qj, bool tri_a, bool tri_b, NearSum& J, NearVir& V)
 {
-    const f2 dx = add2(I.x, xj), dy = add2(I.y, yj), dz = add2(I.z, zj);
+    const f2 dx = add2(pk(A.x, A.y), xj), dy = add2(pk(A.z, A.w), yj), dz = add2(pk(B.x, B.y), zj);
     const f2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-    const float r2a = r2.x, r2b = r2.y;
-    bool ina = r2a < a.rc2, inb = r2b < a.rc2;
+    bool ina = r2.x < a.rc2, inb = r2.y < a.rc2;
     if (TRI) {
         ina = ina && tri_a;
         inb = inb && tri_b;
     }
     if (!__any_sync(0xffffffffu, ina || inb)) return;
     // pairs outside r_c (or not counted) get r^2 = r_c^2 and charge 0 on both sides: finite, adds 0
-    const float ua = ina ? r2a : a.rc2, ub = inb ? r2b : a.rc2;
+    const float ua = ina ? r2.x : a.rc2, ub = inb ? r2.y : a.rc2;
     const f2 u = pk(ua, ub);
-    f2 ri = pk(rsqrt_ftz(ua), rsqrt_ftz(ub));
-    if (USR_NEAR_NEWTON) ri = mul2(ri, fma2(mul2(mul2(u, ri), ri), dup(-0.5f), dup(1.5f)));
-    // pn = -F(u) and its derivative chain, so that N = 1/r + pn needs no sign change
-    const f2 s = fma2(u, dup(a.two_over_rc2), dup(-1.0f));
-    f2 pn = dup(a.npoly[DEG]), dpn = pn;
-    pn = fma2(pn, s, dup(a.npoly[DEG - 1]));
+    const f2 ri = pk(rsqrt_ftz(ua), rsqrt_ftz(ub));
+    // pn = -F(u), d2 = 2 dF/du: two Horner chains side by side, so that N = 1/r + pn needs no sign change
+    const f2 s = fma2(u, a.sfac, dup(-1.0f));
+    f2 pn = a.npoly[DEG], d2 = a.dpoly[DEG - 1];
     #pragma unroll
-    for (int d = DEG - 2; d >= 0; --d) {
-        dpn = fma2(dpn, s, pn);
-        pn = fma2(pn, s, dup(a.npoly[d]));
+    for (int d = DEG - 1; d >= 0; --d) {
+        pn = fma2(pn, s, a.npoly[d]);
+        if (d > 0) d2 = fma2(d2, s, a.dpoly[d - 1]);
     }
-    f2 d2 = mul2(dpn, dup(a.nd2fac));                                     // 2 dF/du
     const int nexp = NEXP >= 0 ? NEXP : a.n_explicit;
     #pragma unroll
     for (int e = 0; e < nexp; ++e) {
-        const f2 t = mul2(u, dup(a.el2[e]));
-        const f2 ggn = mul2(pk(exp2_ftz(t.x), exp2_ftz(t.y)), dup(a.nea[e]));   // minus the Gaussian
-        pn = add2(pn, ggn);
-        d2 = fma2(ggn, dup(a.nne2[e]), d2);
+        const f2 t = mul2(u, a.el2[e]);
+        const f2 x = pk(exp2_ftz(t.x), exp2_ftz(t.y));
+        pn = fma2(x, a.nea[e], pn);
+        d2 = fma2(x, a.dea[e], d2);
     }
     const f2 nr = add2(ri, pn);                                           // N(r) = 1/r - F
     const f2 g = fma2(mul2(ri, ri), ri, d2);                              // -N'(r) / r
-    const float qia = I.q.x, qib = I.q.y;
     const f2 Qj = pk(ina ? qj : 0.f, inb ? qj : 0.f);
-    const f2 Qi = pk(ina ? qia : 0.f, inb ? qib : 0.f);
+    const f2 Qi = pk(ina ? B.z : 0.f, inb ? B.w : 0.f);
     const f2 gi = mul2(g, Qj);
-    I.fx = fma2(gi, dx, I.fx);
-    I.fy = fma2(gi, dy, I.fy);
-    I.fz = fma2(gi, dz, I.fz);
-    I.ph = fma2(nr, Qj, I.ph);
+    I.x = fma2(gi, dx, I.x);
+    I.y = fma2(gi, dy, I.y);
+    I.z = fma2(gi, dz, I.z);
+    I.p = fma2(nr, Qj, I.p);
     const f2 gj = mul2(g, Qi);
-    fjx = fma2(gj, dx, fjx);
-    fjy = fma2(gj, dy, fjy);
-    fjz = fma2(gj, dz, fjz);
-    fjp = fma2(nr, Qi, fjp);
+    J.x = fma2(gj, dx, J.x);
+    J.y = fma2(gj, dy, J.y);
+    J.z = fma2(gj, dz, J.z);
+    J.p = fma2(nr, Qi, J.p);
     if (VIR) {
         // q_i q_j g d (x) d over the pairs (each unordered pair once)
-        const f2 w = mul2(gi, I.q);
+        const f2 w = mul2(gi, pk(B.z, B.w));
         const f2 wx = mul2(w, dx), wy = mul2(w, dy);
         V.xx = fma2(wx, dx, V.xx);
         V.xy = fma2(wx, dy, V.xy);
@@ -189,137 +179,197 @@ __device__ __forceinline__ void pair_step(const NearArgs& a, NearI& I, f2 xj, f2
 }
 
 /*
- * The half-shell neighbour cells of a work unit: offsets nb = 13 (the own cell) .. 26 split into
- * kNearSplits ranges of about equal work (the own cell counts half: only j-clusters from the group's
- * first on).
+ * The half-shell neighbour cells of a work unit: offsets nb = 13 (the own cell) .. 26 split into kNearSplits
+ * ranges of kSplitCells cells.
  */
-constexpr int kNearSplits = 4;
-__constant__ int kSplitLo[kNearSplits] = {13, 17, 20, 23};
-__constant__ int kSplitHi[kNearSplits] = {17, 20, 23, 27};
+constexpr int kNearSplits = 7, kSplitCells = (14 + kNearSplits - 1) / kNearSplits;
+
+/* A warp's shared memory: its group's i atoms in the paired layout (per cluster four 32-byte rows gi: x, x', y,
+   y', z, z', q, q' of atoms gi and gi + 4), their boxes, and the unit's neighbour cells: candidate t of cell k
+   (end[k - 1] <= t < end[k]) is cluster off[k] + t, at image shift sh[k]. */
+template <int GI>
+struct NearShared {
+    float4 ipos[GI][8];
+    float4 box[GI][2];
+    float4 sh[kSplitCells];
+    int off[kSplitCells], end[kSplitCells];
+};
+
+/* The group of work unit u into d (a warp's next unit, or none when u >= units). */
+__device__ __forceinline__ int near_next(const ClusterList& L, const NearArgs& a, int u, int units, int4& d)
+{
+    if (u < units) d = L.gdesc[u / kNearSplits];
+    return u;
+}
 
 /*
- * One work unit: group `grp` (its GI clusters' i atoms) against the j-clusters of the neighbour
- * offsets nb0 .. nb1 - 1.  Adds the i- and j-side parts to acc; VIR: writes the unit's pair virial
- * sum_pairs d (x) f (six FP64 values) to vir.
+ * One work unit: group d = (first cluster, cell, clusters) (its GI clusters' i atoms) against the j-clusters of
+ * the neighbour offsets nb0 .. nb1 - 1.  Adds the i- and j-side parts to acc; VIR: writes the unit's pair virial
+ * sum_pairs d (x) f (six FP64 values) to vir.  Takes the warp's next unit from the queue on the way (`next`) and
+ * loads its group into dn, so that those two dependent reads are not waited for.
  */
 template <int GI, int DEG, int NEXP, bool VIR>
-__device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& a, int grp, int nb0, int nb1,
-                                          float4 (*sbox)[2], unsigned long long* __restrict__ acc,
-                                          double* __restrict__ vir, int* __restrict__ status)
+__device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& a, int4 d, int nb0, int nb1,
+                                          NearShared<GI>& S, unsigned long long* __restrict__ acc,
+                                          double* __restrict__ vir, int* __restrict__ queue, int units, int& next,
+                                          int4& dn, int* __restrict__ status)
 {
+    static_assert(GI * 8 == 32, "one lane per i atom of the group");
     const int lane = threadIdx.x & 31;
     const int ncx = a.box.nc[0], ncy = a.box.nc[1], ncz = a.box.nc[2];
-    if (!USR_IN_BOUNDS(grp, a.max_groups, status)) return;
-    const int c0 = L.gfirst[grp];
-    if (!USR_IN_BOUNDS(c0, a.max_clusters, status)) return;
-    const int cell = L.ccell[c0];
-    const int ni = min(GI, (L.pstart[cell + 1] >> 3) - c0);
-    if (!USR_IN_BOUNDS(c0 + ni - 1, a.max_clusters, status)) return;
+    const int c0 = d.x, cell = d.y, ni = d.z;
+    int ticket = 0;
+    if (lane == 0) ticket = atomicAdd(queue, 1);
     const int jl = lane & 7, gi = lane >> 3;
-    NearI I[GI];
-    #pragma unroll
-    for (int k = 0; k < GI; ++k) {
-        I[k].fx = I[k].fy = I[k].fz = I[k].ph = dup(0.f);
-        if (k < ni) {
-            // padding rows (index -1) move to +1e7 as i atoms, far from every j position
-            const bool va = L.cidx[(c0 + k) * 8 + gi] >= 0, vb = L.cidx[(c0 + k) * 8 + gi + 4] >= 0;
-            // group gi of the paired layout: (x, x', y, y') and (z, z', q, q') of atoms gi and gi + 4
-            const float4 A = L.cpos[(c0 + k) * 8 + 2 * gi], B = L.cpos[(c0 + k) * 8 + 2 * gi + 1];
-            I[k].x = pk(va ? A.x : 1.0e7f, vb ? A.y : 1.0e7f);
-            I[k].y = pk(va ? A.z : 1.0e7f, vb ? A.w : 1.0e7f);
-            I[k].z = pk(va ? B.x : 1.0e7f, vb ? B.y : 1.0e7f);
-            I[k].q = pk(B.z, B.w);
-        } else {
-            I[k].x = I[k].y = I[k].z = I[k].q = dup(0.f);   // never stepped: its mask bit is never set
-        }
+    const int ncells = nb1 - nb0;
+    {
+        // the group's atoms, one per lane; padding rows (near -1e6) move to +1e7, far from every j position
+        float4 p = make_float4(1.0e7f, 1.0e7f, 1.0e7f, 0.f);
+        if (gi < ni) p = L.cpos[c0 * 8 + lane];
+        if (p.x < -5.0e5f) p = make_float4(1.0e7f, 1.0e7f, 1.0e7f, 0.f);
+        float* row = reinterpret_cast<float*>(&S.ipos[gi][2 * (jl & 3)]) + (jl >> 2);
+        row[0] = p.x;
+        row[2] = p.y;
+        row[4] = p.z;
+        row[6] = p.w;
     }
     if (lane < 2 * GI) {
         const int k = lane >> 1;
         float4 v;
         if (k < ni) v = (lane & 1) ? L.bbhi[c0 + k] : L.bblo[c0 + k];
         else v = (lane & 1) ? make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f) : make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
-        sbox[k][lane & 1] = v;
+        S.box[k][lane & 1] = v;
     }
-    __syncwarp();
-    NearVir V;
-    V.xx = V.yy = V.zz = V.xy = V.xz = V.yz = dup(0.f);
-    const bool tri_a = jl > gi, tri_b = jl > gi + 4;
-    const int cx = cell % ncx, cy = (cell / ncx) % ncy, cz = cell / (ncx * ncy);
-    const float* cf = reinterpret_cast<const float*>(L.cpos);
-    // the lane's j atom jl in the paired cluster layout: group jl % 4, half jl / 4
-    const int joff = 8 * (jl & 3) + (jl >> 2);
-    const bool b1 = (lane & 16) != 0, b0 = (lane & 8) != 0;
-    for (int nb = nb0; nb < nb1; ++nb) {
+    int total;
+    {
+        // lane k < ncells: neighbour cell nb0 + k, its image shift and cluster range
+        const int cx = cell % ncx, cy = (cell / ncx) % ncy, cz = cell / (ncx * ncy);
+        const int nb = nb0 + min(lane, ncells - 1);
         int nx = cx + nb % 3 - 1, ny = cy + (nb / 3) % 3 - 1, nz = cz + nb / 9 - 1;
         float sx = 0.f, sy = 0.f, sz = 0.f;
         if (nx < 0) { nx += ncx; sx = -a.box.L[0]; } else if (nx >= ncx) { nx -= ncx; sx = a.box.L[0]; }
         if (ny < 0) { ny += ncy; sy = -a.box.L[1]; } else if (ny >= ncy) { ny -= ncy; sy = a.box.L[1]; }
         if (nz < 0) { nz += ncz; sz = -a.box.L[2]; } else if (nz >= ncz) { nz -= ncz; sz = a.box.L[2]; }
         const int nc = (nz * ncy + ny) * ncx + nx;
-        const bool own = nb == 13;
-        const int jc0 = own ? c0 : L.pstart[nc] >> 3, jc1 = L.pstart[nc + 1] >> 3;
-        for (int jb = jc0; jb < jc1; jb += 32) {
-            const int jc = jb + lane;
-            unsigned int m = 0;
-            if (jc < jc1 && USR_IN_BOUNDS(jc, a.max_clusters, status)) {
-                const float4 lo = L.bblo[jc], hi = L.bbhi[jc];
-                const float lx = __fadd_rn(lo.x, sx), ly = __fadd_rn(lo.y, sy), lz = __fadd_rn(lo.z, sz);
-                const float hx = __fadd_rn(hi.x, sx), hy = __fadd_rn(hi.y, sy), hz = __fadd_rn(hi.z, sz);
+        const int jc0 = nb == 13 ? c0 : L.pstart[nc] >> 3, jc1 = L.pstart[nc + 1] >> 3;
+        const int cnt = lane < ncells ? jc1 - jc0 : 0;
+        int inc = cnt;
+        #pragma unroll
+        for (int o = 1; o < kSplitCells; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        total = __shfl_sync(0xffffffffu, inc, kSplitCells - 1);
+        if (lane < kSplitCells) {
+            S.sh[lane] = make_float4(sx, sy, sz, 0.f);
+            S.off[lane] = jc0 - (inc - cnt);
+            S.end[lane] = inc;
+        }
+    }
+    __syncwarp();
+    NearSum I[GI];
+    #pragma unroll
+    for (int k = 0; k < GI; ++k) I[k].x = I[k].y = I[k].z = I[k].p = dup(0.f);
+    NearVir V;
+    V.xx = V.yy = V.zz = V.xy = V.xz = V.yz = dup(0.f);
+    const bool tri_a = jl > gi, tri_b = jl > gi + 4;
+    const bool b1 = (lane & 16) != 0, b0 = (lane & 8) != 0;
+    if (total == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn);
+    // clusters of the unit's own cell come first: candidate t < GI is cluster c0 + t, one of the group's own
+    const int nown = nb0 == 13 ? ni : 0;
+    int ends[kSplitCells];                 // uniform copies
+    #pragma unroll
+    for (int k = 0; k < kSplitCells; ++k) ends[k] = S.end[k];
+    auto cell_of = [&](int t) {
+        int k = 0;
+        #pragma unroll
+        for (int c = 0; c + 1 < kSplitCells; ++c) k += t >= ends[c];
+        return k;
+    };
+    for (int tb = 0; tb < total; tb += 32) {
+        unsigned int m = 0;
+        {
+            const int t = tb + lane;
+            const int k = cell_of(t);
+            if (t < total) {
+                const int jc = S.off[k] + t;
+                if (USR_IN_BOUNDS(jc, a.max_clusters, status)) {
+                    const float4 lo = L.bblo[jc], hi = L.bbhi[jc], sh = S.sh[k];
+                    const float lx = __fadd_rn(lo.x, sh.x), ly = __fadd_rn(lo.y, sh.y), lz = __fadd_rn(lo.z, sh.z);
+                    const float hx = __fadd_rn(hi.x, sh.x), hy = __fadd_rn(hi.y, sh.y), hz = __fadd_rn(hi.z, sh.z);
+                    #pragma unroll
+                    for (int i = 0; i < GI; ++i) {
+                        const float4 blo = S.box[i][0], bhi = S.box[i][1];
+                        // gap between the boxes, rounded like a pair distance
+                        const float gx = fmaxf(0.f, fmaxf(__fsub_rn(lx, bhi.x), __fsub_rn(blo.x, hx)));
+                        const float gy = fmaxf(0.f, fmaxf(__fsub_rn(ly, bhi.y), __fsub_rn(blo.y, hy)));
+                        const float gz = fmaxf(0.f, fmaxf(__fsub_rn(lz, bhi.z), __fsub_rn(blo.z, hz)));
+                        if (__fmaf_rn(gz, gz, __fmaf_rn(gy, gy, __fmul_rn(gx, gx))) < a.rc2) m |= 1u << i;
+                    }
+                    // own cell: i-cluster c0 + k meets j-clusters from c0 + k on
+                    if (t < nown) m &= (2u << t) - 1u;
+                }
+            }
+        }
+        if (tb == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn);
+        unsigned int bal = __ballot_sync(0xffffffffu, m != 0);
+        if (!bal) continue;
+        // the surviving j-clusters; the next one's atoms are loaded while this one's steps run
+        int t = __ffs(bal) - 1;
+        int tc = tb + t;
+        int k = cell_of(tc);
+        int jcl = S.off[k] + tc;
+        float4 pj = L.cpos[jcl * 8 + jl];
+        for (;;) {
+            bal &= bal - 1;
+            const float4 sh = S.sh[k];
+            const unsigned int mk = __shfl_sync(0xffffffffu, m, t);
+            const int jcur = jcl;
+            const bool own = tc < nown;
+            // minus the image position, -(x_j + shift): d = x_i + that, the same number as x_i - (x_j + shift)
+            const f2 xj = dup(-__fadd_rn(pj.x, sh.x)), yj = dup(-__fadd_rn(pj.y, sh.y)), zj = dup(-__fadd_rn(pj.z, sh.z));
+            const float qj = pj.w;
+            const int own_k = tc;
+            if (bal) {
+                t = __ffs(bal) - 1;
+                tc = tb + t;
+                k = cell_of(tc);
+                jcl = S.off[k] + tc;
+                pj = L.cpos[jcl * 8 + jl];
+            }
+            NearSum J;
+            J.x = J.y = J.z = J.p = dup(0.f);
+            if (own) {
+                // the j-cluster is one of the group's own: that step counts j after i only
                 #pragma unroll
-                for (int k = 0; k < GI; ++k) {
-                    const float4 blo = sbox[k][0], bhi = sbox[k][1];
-                    // gap between the boxes, rounded like a pair distance
-                    const float gx = fmaxf(0.f, fmaxf(__fsub_rn(lx, bhi.x), __fsub_rn(blo.x, hx)));
-                    const float gy = fmaxf(0.f, fmaxf(__fsub_rn(ly, bhi.y), __fsub_rn(blo.y, hy)));
-                    const float gz = fmaxf(0.f, fmaxf(__fsub_rn(lz, bhi.z), __fsub_rn(blo.z, hz)));
-                    if (__fmaf_rn(gz, gz, __fmaf_rn(gy, gy, __fmul_rn(gx, gx))) < a.rc2) m |= 1u << k;
-                }
-                // own cell: i-cluster c0 + k meets j-clusters from c0 + k on
-                if (own && jc - c0 < GI) m &= (2u << (jc - c0)) - 1u;
+                for (int i = 0; i < GI; ++i)
+                    if (mk & (1u << i)) {
+                        const float4 A = S.ipos[i][2 * gi], B = S.ipos[i][2 * gi + 1];
+                        if (own_k == i)
+                            pair_step<DEG, NEXP, VIR, true>(a, A, B, I[i], xj, yj, zj, qj, tri_a, tri_b, J, V);
+                        else
+                            pair_step<DEG, NEXP, VIR, false>(a, A, B, I[i], xj, yj, zj, qj, tri_a, tri_b, J, V);
+                    }
+            } else {
+                #pragma unroll
+                for (int i = 0; i < GI; ++i)
+                    if (mk & (1u << i)) {
+                        const float4 A = S.ipos[i][2 * gi], B = S.ipos[i][2 * gi + 1];
+                        pair_step<DEG, NEXP, VIR, false>(a, A, B, I[i], xj, yj, zj, qj, tri_a, tri_b, J, V);
+                    }
             }
-            unsigned int bal = __ballot_sync(0xffffffffu, m != 0);
-            while (bal) {
-                const int t = __ffs(bal) - 1;
-                bal &= bal - 1;
-                const int jcl = jb + t;
-                const unsigned int mk = __shfl_sync(0xffffffffu, m, t);
-                const float* pj = cf + jcl * 32 + joff;
-                // minus the image position, -(x_j + shift): d = x_i + that, the same number as x_i - (x_j + shift)
-                const float xj = -__fadd_rn(pj[0], sx), yj = -__fadd_rn(pj[2], sy), zj = -__fadd_rn(pj[4], sz);
-                const float qj = pj[6];
-                const int sj = L.cidx[jcl * 8 + jl];
-                const f2 xj2 = dup(xj), yj2 = dup(yj), zj2 = dup(zj);
-                f2 fjx = dup(0.f), fjy = dup(0.f), fjz = dup(0.f), fjp = dup(0.f);
-                if (own && jcl - c0 < GI) {
-                    // the j-cluster is one of the group's own: that step counts j after i only
-                    #pragma unroll
-                    for (int k = 0; k < GI; ++k)
-                        if (mk & (1u << k)) {
-                            if (jcl == c0 + k)
-                                pair_step<DEG, NEXP, VIR, true>(a, I[k], xj2, yj2, zj2, qj, tri_a, tri_b, fjx, fjy,
-                                                                fjz, fjp, V);
-                            else
-                                pair_step<DEG, NEXP, VIR, false>(a, I[k], xj2, yj2, zj2, qj, tri_a, tri_b, fjx, fjy,
-                                                                 fjz, fjp, V);
-                        }
-                } else {
-                    #pragma unroll
-                    for (int k = 0; k < GI; ++k)
-                        if (mk & (1u << k))
-                            pair_step<DEG, NEXP, VIR, false>(a, I[k], xj2, yj2, zj2, qj, tri_a, tri_b, fjx, fjy, fjz,
-                                                             fjp, V);
-                }
-                // j-side sums: fold the two i halves, reduce-scatter over the four lanes gi of atom jl
-                const float vx = fjx.x + fjx.y, vy = fjy.x + fjy.y;
-                const float vz = fjz.x + fjz.y, vp = fjp.x + fjp.y;
-                const float r0 = __shfl_xor_sync(0xffffffffu, b1 ? vx : vz, 16);
-                const float r1 = __shfl_xor_sync(0xffffffffu, b1 ? vy : vp, 16);
-                const float k0 = (b1 ? vz : vx) + r0, k1 = (b1 ? vp : vy) + r1;
-                const float r2 = __shfl_xor_sync(0xffffffffu, b0 ? k0 : k1, 8);
-                const float v = (b0 ? k1 : k0) + r2;                           // component gi of atom jl
-                if (sj >= 0 && USR_IN_BOUNDS(sj, a.max_atoms, status))
-                    red_fix(acc + 4 * (size_t)sj + gi, gi < 3 ? -qj * v : v, status);
-            }
+            // j-side sums: fold the two i halves, reduce-scatter over the four lanes gi of atom jl; lane
+            // (jl, gi) ends with component gi, which is accumulator `lane` of the cluster
+            const float vx = J.x.x + J.x.y, vy = J.y.x + J.y.y;
+            const float vz = J.z.x + J.z.y, vp = J.p.x + J.p.y;
+            const float r0 = __shfl_xor_sync(0xffffffffu, b1 ? vx : vz, 16);
+            const float r1 = __shfl_xor_sync(0xffffffffu, b1 ? vy : vp, 16);
+            const float k0 = (b1 ? vz : vx) + r0, k1 = (b1 ? vp : vy) + r1;
+            const float r2 = __shfl_xor_sync(0xffffffffu, b0 ? k0 : k1, 8);
+            const float v = (b0 ? k1 : k0) + r2;
+            if (USR_IN_BOUNDS(jcur, a.max_clusters, status))
+                red_fix(acc + 32 * (size_t)jcur + lane, gi < 3 ? -qj * v : v, status);
+            if (!bal) break;
         }
     }
     // i-side sums: reduce-scatter the 8 values of each cluster (2 atoms x 4 components) over the 8
@@ -328,8 +378,8 @@ __device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& 
     #pragma unroll
     for (int k = 0; k < GI; ++k) {
         if (k >= ni) break;
-        const float va[4] = {I[k].fx.x, I[k].fy.x, I[k].fz.x, I[k].ph.x};
-        const float vb[4] = {I[k].fx.y, I[k].fy.y, I[k].fz.y, I[k].ph.y};
+        const float va[4] = {I[k].x.x, I[k].y.x, I[k].z.x, I[k].p.x};
+        const float vb[4] = {I[k].x.y, I[k].y.y, I[k].z.y, I[k].p.y};
         float w4[4];
         #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -345,11 +395,9 @@ __device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& 
         const float r = __shfl_xor_sync(0xffffffffu, c0b ? w2[0] : w2[1], 1);
         const float v = (c0b ? w2[1] : w2[0]) + r;
         const int comp = jl & 3;
-        const int slot = (c0 + k) * 8 + gi + 4 * (jl >> 2);
-        const int si = L.cidx[slot];
-        const float qi = c2 ? I[k].q.y : I[k].q.x;
-        if (si >= 0 && USR_IN_BOUNDS(si, a.max_atoms, status))
-            red_fix(acc + 4 * (size_t)si + comp, comp < 3 ? qi * v : v, status);
+        const float4 B = S.ipos[k][2 * gi + 1];
+        const float qi = c2 ? B.w : B.z;
+        red_fix(acc + 32 * (size_t)(c0 + k) + 8 * comp + gi + 4 * (jl >> 2), comp < 3 ? qi * v : v, status);
     }
     if (VIR) {
         const f2 vv[6] = {V.xx, V.yy, V.zz, V.xy, V.xz, V.yz};
@@ -363,34 +411,40 @@ __device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& 
         if (lane == 0)
             for (int c6 = 0; c6 < 6; ++c6) vir[c6] = v6[c6];
     }
-    __syncwarp();   // sbox is rewritten by the warp's next unit
+    __syncwarp();   // S is rewritten by the warp's next unit
 }
 
 /*
  * Persistent warps: each takes work units (group, neighbour range) from a queue counter (zeroed by
  * the cell-list scan), full groups first and the partial ones last, until none is left.  The
  * accumulation is integer, so results do not depend on which warp takes which unit.  acc: 4
- * fixed-point accumulators (Fx, Fy, Fz, phi) per sorted atom, zeroed by k_cluster_build.  VIR: unit u
+ * fixed-point accumulators (Fx, Fy, Fz, phi) per cluster slot, zeroed by k_cluster_build.  VIR: unit u
  * writes its pair virial to vir[6 u ..].
  */
 template <int GI, int DEG, int NEXP, bool VIR>
-__global__ void __launch_bounds__(128, USR_NEAR_MINB) k_near_half(ClusterList L, NearArgs a, int* __restrict__ queue,
+__global__ void __launch_bounds__(128, USR_NEAR_MINB) k_near_half(ClusterList L, const __grid_constant__ NearArgs a,
+                                                                    int* __restrict__ queue,
                                                                     unsigned long long* __restrict__ acc,
                                                                     double* __restrict__ vir, int* __restrict__ status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
-    __shared__ float4 sbox[4][GI][2];
+    __shared__ NearShared<GI> S[4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ncell = a.box.nc[0] * a.box.nc[1] * a.box.nc[2];
     const int units = kNearSplits * (L.gfull[ncell] + L.gpart[ncell]);
-    for (;;) {
-        int u = 0;
-        if (lane == 0) u = atomicAdd(queue, 1);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= units) break;
-        const int grp = u / kNearSplits, sub = u - grp * kNearSplits;
-        near_unit<GI, DEG, NEXP, VIR>(L, a, grp, kSplitLo[sub], kSplitHi[sub], sbox[warp], acc,
-                                      VIR ? vir + 6 * (size_t)u : nullptr, status);
+    int u = 0;
+    if (lane == 0) u = atomicAdd(queue, 1);
+    int4 d = make_int4(0, 0, 0, 0);
+    u = near_next(L, a, __shfl_sync(0xffffffffu, u, 0), units, d);
+    while (u < units) {
+        const int sub = u % kNearSplits, nb0 = 13 + sub * kSplitCells, nb1 = min(27, nb0 + kSplitCells);
+        if (!USR_IN_BOUNDS(d.x + d.z - 1, a.max_clusters, status)) return;
+        int next = units;
+        int4 dn = d;
+        near_unit<GI, DEG, NEXP, VIR>(L, a, d, nb0, nb1, S[warp], acc, VIR ? vir + 6 * (size_t)u : nullptr, queue,
+                                      units, next, dn, status);
+        u = next;
+        d = dn;
     }
 }
 
@@ -402,7 +456,7 @@ __global__ void __launch_bounds__(128, USR_NEAR_MINB) k_near_half(ClusterList L,
  * single-precision predicate d = x_i - (x_j + shift), evaluated from i's side;
  * count and the sum of splitmix64 of the partners' caller indices.
  */
-__global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, const int* __restrict__ perm, NearArgs a,
+__global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, NearArgs a,
                                                      int* __restrict__ count, unsigned long long* __restrict__ hash,
                                                      int* __restrict__ status)
 {
@@ -413,9 +467,7 @@ __global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, const int* _
     if (ic >= ncl || !USR_IN_BOUNDS(ic, a.max_clusters, status)) return;
     const int il = lane >> 2, g = lane & 3;
     const int islot = ic * 8 + il;
-    const float* cf = reinterpret_cast<const float*>(L.cpos);
-    const int io = ic * 32 + 8 * (il & 3) + (il >> 2);
-    const float4 pi = make_float4(cf[io], cf[io + 2], cf[io + 4], cf[io + 6]);
+    const float4 pi = L.cpos[islot];
     const f2 pix = dup(pi.x), piy = dup(pi.y), piz = dup(pi.z);
     const float4 blo = L.bblo[ic], bhi = L.bbhi[ic];
     const int c = L.ccell[ic];
@@ -446,21 +498,20 @@ __global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, const int* _
                 const int k = __ffs(m) - 1;
                 m &= m - 1;
                 const int jcl = jb + k;
-                const float4 A = L.cpos[jcl * 8 + 2 * g];     // (x_g, x_g+4, y_g, y_g+4)
-                const float4 B = L.cpos[jcl * 8 + 2 * g + 1]; // (z_g, z_g+4, q_g, q_g+4)
-                const f2 dx = sub2(pix, add2(pk(A.x, A.y), sx2));
-                const f2 dy = sub2(piy, add2(pk(A.z, A.w), sy2));
-                const f2 dz = sub2(piz, add2(pk(B.x, B.y), sz2));
+                const float4 A = L.cpos[jcl * 8 + g], B = L.cpos[jcl * 8 + 4 + g];
+                const f2 dx = sub2(pix, add2(pk(A.x, B.x), sx2));
+                const f2 dy = sub2(piy, add2(pk(A.y, B.y), sy2));
+                const f2 dz = sub2(piz, add2(pk(A.z, B.z), sz2));
                 const f2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
                 const float r2a = r2.x, r2b = r2.y;
                 const bool self = nb == 13 && jcl == ic;
                 if (r2a < a.rc2 && !(self && g == il)) {
                     ++cnt;
-                    h += mix64((unsigned long long)perm[L.cidx[jcl * 8 + g]]);
+                    h += mix64((unsigned long long)L.cperm[jcl * 8 + g]);
                 }
                 if (r2b < a.rc2 && !(self && g + 4 == il)) {
                     ++cnt;
-                    h += mix64((unsigned long long)perm[L.cidx[jcl * 8 + 4 + g]]);
+                    h += mix64((unsigned long long)L.cperm[jcl * 8 + 4 + g]);
                 }
             }
         }
@@ -470,9 +521,8 @@ __global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, const int* _
         cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         h += __shfl_xor_sync(0xffffffffu, h, o);
     }
-    const int si = L.cidx[islot];
-    if (g == 0 && si >= 0) {
-        const int ci = perm[si];
+    const int ci = L.cperm[islot];
+    if (g == 0 && ci >= 0) {
         if (USR_IN_BOUNDS(ci, a.max_atoms, status)) {
             count[ci] = cnt;
             hash[ci] = h;
@@ -571,11 +621,11 @@ void launch_near(int max_groups, int deg, const ClusterList& L, const NearArgs& 
 #undef USR_NEAR_DEG
 }
 
-void launch_pairs(int max_clusters, const ClusterList& L, const int* perm, const NearArgs& a, int* count,
+void launch_pairs(int max_clusters, const ClusterList& L, const NearArgs& a, int* count,
                   unsigned long long* hash, int* status, cudaStream_t st)
 {
     const int blocks = (max_clusters + 3) / 4;
-    k_pairs_count<<<blocks, 128, 0, st>>>(L, perm, a, count, hash, status);
+    k_pairs_count<<<blocks, 128, 0, st>>>(L, a, count, hash, status);
 }
 
 }  // namespace usr

@@ -116,7 +116,7 @@ struct SpreadShared {
    TF32 (1) or BF16 (2).  rho32: FP32 copy beside a split (may be null). */
 template <int S, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4* __restrict__ pos,
-                                                        const int* __restrict__ cell_start, GridArgs g, int P,
+                                                        const int* __restrict__ pstart, GridArgs g, int P,
                                                         int bricks_x, int bricks_y, int bricks, int out,
                                                         void* __restrict__ rho, void* __restrict__ rho_lo,
                                                         float* __restrict__ rho32, double* __restrict__ partial,
@@ -214,15 +214,15 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         const int runs = nz * ny * npx;
         int head = 0, count = 0, turn = 0;
         for (int rb = 0; rb < runs; rb += 32) {
-            // lane = one run of cells: its first sorted atom, length and image shift (grid points, from the brick)
+            // lane = one run of cells: its first slot, length and image shift (grid points, from the brick)
             int first = 0, cnt = 0, sx = 0, sy = 0, sz = 0;
             const int id = rb + lane;
             if (id < runs) {
                 const int cyu = c0[1] + id / npx % ny, czu = c0[2] + id / (npx * ny), kx = px + id % npx;
                 const int qy = floor_div(cyu, ncy), qz = floor_div(czu, ncz);
                 const int row = ((czu - qz * ncz) * ncy + (cyu - qy * ncy)) * ncx;
-                first = cell_start[row + max(c0[0] - kx * ncx, 0)];
-                cnt = cell_start[row + min(c1[0] - kx * ncx, ncx - 1) + 1] - first;
+                first = pstart[row + max(c0[0] - kx * ncx, 0)];
+                cnt = pstart[row + min(c1[0] - kx * ncx, ncx - 1) + 1] - first;
                 sx = kx * n0 - ox - H + 1;
                 sy = qy * n1 - oy - H + 1;
                 sz = qz * n2 - oz - H + 1;
@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                 if (base + lane < rc) next = pos[rf + base + lane];
                 for (; base < rc; base += 32 * S) {
                     const float4 p = next;
-                    bool ok = base + lane < rc && USR_IN_BOUNDS(rf + base + lane, g.max_atoms, status);
+                    // a padding slot lies near -1e6
+                    bool ok = base + lane < rc && p.x > -5.0e5f && USR_IN_BOUNDS(rf + base + lane, g.max_slots, status);
                     if (base + 32 * S + lane < rc) next = pos[rf + base + 32 * S + lane];
                     const float ux = p.x * g.box.gs[0], uy = p.y * g.box.gs[1], uz = p.z * g.box.gs[2];
                     const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
@@ -249,8 +250,10 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                     const unsigned int bal = __ballot_sync(0xffffffffu, ok);
                     if (ok) {
                         const int q = (head + count + __popc(bal & ((1u << lane) - 1u))) & (kQueue - 1);
-                        W.f[q] = make_float4(grid_frac(g.box, 0, p.x, fx), grid_frac(g.box, 1, p.y, fy),
-                                             grid_frac(g.box, 2, p.z, fz), p.w);
+                        // (BF16 operands keep nothing of the fraction's last digits)
+                        W.f[q] = out == 2 ? make_float4(ux - fx, uy - fy, uz - fz, p.w)
+                                          : make_float4(grid_frac(g.box, 0, p.x, fx), grid_frac(g.box, 1, p.y, fy),
+                                                        grid_frac(g.box, 2, p.z, fz), p.w);
                         W.b[q] = (b0 + 32) | (b1 + 32) << 8 | (b2 + 32) << 16;
                     }
                     count += __popc(bal);
@@ -387,13 +390,13 @@ int spread_ctas(const int* n)
     return (bricks_of(n) + nb - 1) / nb;
 }
 
-void launch_spread(int P, const float4* spos, const int* cell_start, const GridArgs& g, int split, void* rho,
+void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, void* rho,
                    void* rho_lo, float* rho32, double* partial, unsigned int* counter, double* mean, int* status,
                    cudaStream_t st)
 {
     const int bx = bricks_along(g.box.n[0], kBrickX), by = bricks_along(g.box.n[1], kBrick);
 #define USR_SPREAD(S, W)                                                                                           \
-    launch_pdl(k_spread<S, W>, spread_ctas(g.box.n), 32 * W, 0, st, spos, cell_start, g, P, bx, by,                 \
+    launch_pdl(k_spread<S, W>, spread_ctas(g.box.n), 32 * W, 0, st, L.cpos, L.pstart, g, P, bx, by,                 \
                bricks_of(g.box.n), split, rho, rho_lo, rho32, partial, counter, mean, status)
     switch (splits_of(g.box.n)) {
         case 1: USR_SPREAD(1, kSpreadWarps); break;

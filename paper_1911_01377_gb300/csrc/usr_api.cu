@@ -68,11 +68,12 @@ struct usr_ctx {
     int *d_count = nullptr, *d_cell_of = nullptr, *d_slot = nullptr, *d_cell_start = nullptr;
     int *d_unsorted = nullptr, *d_perm = nullptr, *d_status = nullptr;
     float4 *d_wpos = nullptr, *d_spos = nullptr;
-    unsigned long long* d_nacc = nullptr;   // near part, 4 fixed-point sums per sorted atom
+    unsigned long long* d_nacc = nullptr;   // near part, 4 fixed-point sums per cluster slot
     // 8-atom clusters of the pair kernel (padded layout)
     int max_clusters = 0, max_groups = 0;
-    int *d_pstart = nullptr, *d_cidx = nullptr, *d_ccell = nullptr, *d_gfull = nullptr, *d_gpart = nullptr;
-    int *d_gfirst = nullptr, *d_queue = nullptr;
+    int *d_pstart = nullptr, *d_cperm = nullptr, *d_ccell = nullptr, *d_gfull = nullptr, *d_gpart = nullptr;
+    int4* d_gdesc = nullptr;
+    int* d_queue = nullptr;
     float4 *d_cpos = nullptr, *d_bblo = nullptr, *d_bbhi = nullptr;
     // grids and convolution tables
     float *d_rho = nullptr, *d_X = nullptr, *d_Y = nullptr, *d_psi = nullptr;
@@ -110,13 +111,13 @@ struct usr_ctx {
     cudaEvent_t stage_ev = nullptr;
     // host-buffer staging and inspection
     float4 *d_in = nullptr, *d_out = nullptr, *d_near_dbg = nullptr, *d_far_dbg = nullptr;
-    float4* d_far4 = nullptr;      // far part per sorted atom (gather -> combination)
+    float4* d_far4 = nullptr;      // far part per cluster slot (gather -> combination)
     bool keep_parts = false;
     bool inject_timeout = false;
     int near_ctas_per_sm = USR_NEAR_CTAS;   // persistent pair-kernel CTAs per SM (0: as many as fit)
     bool parts_valid = false;
-    // the far chain (spread, convolutions, psi mean) runs on `side`, a high-priority stream forked from and
-    // joined back to the caller's stream, while the pair kernel runs on the caller's stream
+    // the pair kernel runs on `side`, a stream forked from and joined back to the caller's, on which the far chain
+    // (spread, convolutions, gather) runs
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // profiling: stage boundary events (see usr_stage_times)
@@ -146,8 +147,8 @@ usr_status dalloc(T** p, size_t count)
 void free_all(usr_ctx* c)
 {
     void* ptrs[] = {c->d_count, c->d_cell_of, c->d_slot, c->d_cell_start, c->d_unsorted, c->d_perm, c->d_status,
-                    c->d_pstart, c->d_cidx, c->d_ccell, c->d_cpos, c->d_bblo, c->d_bbhi,
-                    c->d_wpos, c->d_spos, c->d_nacc, c->d_gfull, c->d_gpart, c->d_gfirst, c->d_queue, c->d_rho, c->d_X, c->d_Y, c->d_psi, c->d_Bx, c->d_Ay,
+                    c->d_pstart, c->d_cperm, c->d_ccell, c->d_cpos, c->d_bblo, c->d_bbhi,
+                    c->d_wpos, c->d_spos, c->d_nacc, c->d_gfull, c->d_gpart, c->d_gdesc, c->d_queue, c->d_rho, c->d_X, c->d_Y, c->d_psi, c->d_Bx, c->d_Ay,
                     c->d_Az, c->d_wx, c->d_wy, c->d_wz, c->d_spread_partial, c->d_mean, c->d_gather_partial,
                     c->d_energy, c->d_netq, c->d_counters, c->d_in, c->d_out, c->d_near_dbg, c->d_far_dbg, c->d_far4,
                     c->d_psi_mean, c->d_ktab};
@@ -212,7 +213,7 @@ void tc_shape(usr::ConvTcArgs& a, int n_out, int K, bool bf16, long long ctas_m)
     a.cols = (n_out + a.ntiles - 1) / a.ntiles;
     a.NT = ((a.cols + 1 + 15) / 16) * 16;
     a.tmem_cols = 32;
-    while (a.tmem_cols < 2 * a.NT) a.tmem_cols *= 2;     // two accumulators
+    while (a.tmem_cols < (bf16 ? 1 : 2) * a.NT) a.tmem_cols *= 2;     // TF32: two accumulators
     const int kstage = bf16 ? 64 : 32;
     const int nk = (K + kstage - 1) / kstage;
     const size_t stage = (size_t)(2 * 128 + 2 * a.NT) * 128;
@@ -274,11 +275,11 @@ double usr::plan_device_bytes(const Plan& P)
     const double nsb = spread_ctas(P.n);
     const double ncl = std::floor((na + 7 * ncell + 7) / 8);
     const double nmax = std::max(nx, std::max(ny, nz));
-    double b = 4096 + 4 * (ncell + 1) * 3 + 16 * ncl * 8 + 4 * ncl * 8 + 4 * ncl + 32 * ncl;   // cells, clusters
+    double b = 4096 + 4 * (ncell + 1) * 3 + 16 * ncl * 8 + 4 * ncl * 8 + 4 * ncl + (32 + 256 + 128) * ncl;   // cells, clusters
     b += 8 * (3 * N * nmax + 4 * N);                                               // 1D kernel tables
-    b += na * (4 * 4 + 16 * 7 + 32);                                               // per-atom arrays
+    b += na * (4 * 4 + 16 * 6);                                               // per-atom arrays
     const double ngr = near_max_groups((int)na, (int)ncell);
-    b += 8 * (ncell + 1) + 4 * ngr + 4;                                            // pair-kernel groups
+    b += 8 * (ncell + 1) + 16 * ngr + 4;                                            // pair-kernel groups
     b += 4 * G + 8 * (nsb + kGatherBlocks + 4 * kCombineBlocks) + 8 * 11;
     if (P.p.virial) {   // six FP32 table sets, their inputs, two FP32 grids, warp slots, FP32 scratch grids
         b += 6 * 4 * N * (nx * nx + ny * ny + nz * nz + nx + ny + nz) + 6 * 8 * (3 * N * nmax + 4 * N);
@@ -433,12 +434,12 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     ENSURE(c->d_cell_start, i4 * (c->ncell + 1));
     ENSURE(c->d_pstart, i4 * (c->ncell + 1));
     ENSURE(c->d_cpos, f4 * ncl * 8);
-    ENSURE(c->d_cidx, i4 * ncl * 8);
+    ENSURE(c->d_cperm, i4 * ncl * 8);
     ENSURE(c->d_ccell, i4 * ncl);
     ENSURE(c->d_gfull, i4 * (c->ncell + 1));
     ENSURE(c->d_gpart, i4 * (c->ncell + 1));
     ENSURE(c->d_queue, i4);
-    ENSURE(c->d_gfirst, i4 * c->max_groups);
+    ENSURE(c->d_gdesc, sizeof(int4) * c->max_groups);
     ENSURE(c->d_bblo, f4 * ncl);
     ENSURE(c->d_bbhi, f4 * ncl);
     ENSURE(c->d_cell_of, i4 * na);
@@ -448,12 +449,12 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     ENSURE(c->d_status, i4);
     ENSURE(c->d_wpos, f4 * na);
     ENSURE(c->d_spos, f4 * na);
-    ENSURE(c->d_nacc, sizeof(unsigned long long) * 4 * na);
+    ENSURE(c->d_nacc, sizeof(unsigned long long) * 32 * ncl);
     ENSURE(c->d_psi, fl * G);
     ENSURE(c->d_spread_partial, db * nsb);
     ENSURE(c->d_mean, db);
     ENSURE(c->d_gather_partial, db * (usr::kGatherBlocks + 4 * usr::kCombineBlocks));
-    ENSURE(c->d_far4, f4 * na);
+    ENSURE(c->d_far4, f4 * ncl * 8);
     ENSURE(c->d_energy, db * 4);
     ENSURE(c->d_netq, db);
     ENSURE(c->d_counters, sizeof(unsigned int) * 8);
@@ -677,28 +678,24 @@ void fill_args(usr_ctx* c)
     a.max_atoms = c->max_atoms > 0 ? c->max_atoms : 1;
     a.max_clusters = c->max_clusters;
     a.max_groups = c->max_groups;
-    a.rc2 = (float)(P.p.r_c * P.p.r_c);
-    a.two_over_rc2 = (float)(2.0 / (P.p.r_c * P.p.r_c));
+    const double rc2 = P.p.r_c * P.p.r_c;
+    auto dup = [](double v) { return make_float2((float)v, (float)v); };
+    a.rc2 = (float)rc2;
+    a.sfac = dup(2.0 / rc2);
     a.n_explicit = P.n_explicit;
     for (int e = 0; e < P.n_explicit; ++e) {
-        a.ea[e] = (float)P.ea[e];
-        a.einv[e] = (float)P.einv[e];
-        a.el2[e] = (float)(-P.einv[e] * 1.4426950408889634);    // log2(e)
-        a.ne2[e] = (float)(-2.0 * P.einv[e]);
+        a.el2[e] = dup(-P.einv[e] * 1.4426950408889634);    // log2(e)
+        a.nea[e] = dup(-P.ea[e]);
+        a.dea[e] = dup(-2.0 * P.einv[e] * P.ea[e]);
     }
     for (int d = 0; d <= usr::kMaxPolyDeg; ++d) {
-        a.poly[d] = (float)P.poly[d];
-        a.npoly[d] = -a.poly[d];
+        a.npoly[d] = dup(-P.poly[d]);
+        if (d > 0) a.dpoly[d - 1] = dup(4.0 / rc2 * d * P.poly[d]);   // 2 dF/du = 2 (2 / r_c^2) dF/ds
     }
-    for (int e = 0; e < usr::kMaxExplicit; ++e) {
-        a.nea[e] = -a.ea[e];
-        a.nne2[e] = -a.ne2[e];
-    }
-    a.nd2fac = -2.0f * a.two_over_rc2;
     usr::GridArgs& g = c->grid;
     std::memset(&g, 0, sizeof(g));
     g.box = c->boxf;
-    g.max_atoms = c->max_atoms > 0 ? c->max_atoms : 1;
+    g.max_slots = 8 * c->max_clusters;
     for (int ax = 0; ax < 3; ++ax) {
         g.hh[ax] = (float)(P.h[ax] * P.h[ax] / (2.0 * P.sigma_sa[ax] * P.sigma_sa[ax]));
         g.dfac[ax] = (float)(P.h[ax] / (P.sigma_sa[ax] * P.sigma_sa[ax]));
@@ -715,40 +712,28 @@ usr_status check_device(const usr_ctx* c)
     return dev == c->device ? USR_OK : USR_ERR_ARG;
 }
 
-/* Cell list in canonical sorted order (cell ids, counting sort, order by caller index within a cell). */
-void bin_sorted(usr_ctx* c, int n, const float4* xyzq, cudaStream_t st)
-{
-    usr::launch_bin_sorted(n, xyzq, c->boxf, c->ncell, c->d_count, c->d_cell_of, c->d_slot, c->d_wpos,
-                           c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, c->d_unsorted, c->d_perm,
-                           c->d_spos, c->d_status, st);
-}
-
-/* The pair kernels' 8-atom clusters, groups and zeroed accumulators, from the sorted cell list. */
-void build_clusters(usr_ctx* c, int n, cudaStream_t st)
-{
-    usr::launch_clusters(n, c->boxf, c->ncell, c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_gfirst,
-                         c->d_spos, c->d_slot, c->d_cpos, c->d_cidx, c->d_ccell, c->d_bblo, c->d_bbhi, c->d_nacc,
-                         c->max_clusters, c->max_groups, c->d_status, st);
-}
-
+/* Cell list, 8-atom clusters, groups and zeroed accumulators. */
 void bin_and_cluster(usr_ctx* c, int n, const float4* xyzq, cudaStream_t st)
 {
-    bin_sorted(c, n, xyzq, st);
-    build_clusters(c, n, st);
+    usr::launch_bin_list(n, xyzq, c->boxf, c->ncell, c->d_count, c->d_cell_of, c->d_slot, c->d_wpos, c->d_cell_start,
+                         c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, c->d_unsorted, c->d_status, st);
+    usr::launch_clusters(n, c->boxf, c->ncell, c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_gdesc,
+                         c->d_unsorted, c->d_wpos, c->d_slot, c->d_cpos, c->d_cperm, c->d_ccell, c->d_bblo, c->d_bbhi,
+                         c->d_nacc, c->max_clusters, c->max_groups, c->d_status, st);
 }
 
 usr::ClusterList cluster_list(const usr_ctx* c)
 {
     usr::ClusterList L;
     L.cpos = c->d_cpos;
-    L.cidx = c->d_cidx;
+    L.cperm = c->d_cperm;
     L.ccell = c->d_ccell;
     L.bblo = c->d_bblo;
     L.bbhi = c->d_bbhi;
     L.pstart = c->d_pstart;
     L.gfull = c->d_gfull;
     L.gpart = c->d_gpart;
-    L.gfirst = c->d_gfirst;
+    L.gdesc = c->d_gdesc;
     return L;
 }
 
@@ -829,9 +814,9 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
         c->vir_valid = c->vir;
         return USR_OK;
     }
-    // stage boundaries: on the caller's stream 0 start, 1 cell list done, 2 pair kernel done, 9 the
-    // combination may start (the far chain joined), 10 end; on the side stream 3 start, 4 spread done, 5-7
-    // passes x, y, z done, 8 multilevel coarse steps done, 11 far gather done
+    // stage boundaries: on the caller's stream 0 start, 3 cell list done, 4 spread done, 5-7 passes x, y, z done,
+    // 8 multilevel coarse steps done, 11 far gather done, 9 the combination may start (the pair kernel joined),
+    // 10 end; on the side stream 1 pair kernel may start, 2 pair kernel done
     auto mark = [&](int k, cudaStream_t s) {
         if (c->prof == 1 || (c->prof == 2 && (k == 1 || k == 2))) cudaEventRecord(c->ev[k], s);
     };
@@ -839,28 +824,32 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
     mark(0, st);
     {
         NvtxRange r("usr: cell list");
-        bin_sorted(c, n, xyzq, st);
+        bin_and_cluster(c, n, xyzq, st);
     }
-    // fork: the far chain needs only the sorted cell list, so it starts on the side stream while the caller's
-    // stream builds the pair kernel's clusters and then runs the pair kernel
+    // fork: the pair kernel runs on the side stream; the far chain stays on the caller's, where its first kernel
+    // is scheduled as the clusters complete, ahead of the pair kernel's persistent CTAs (which would otherwise
+    // fill the SMs first and leave the whole chain the one slot they spare)
     if (cudaEventRecord(c->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(c->side, c->ev_fork, 0) != cudaSuccess)
         return USR_ERR_CUDA;
-    {
-        NvtxRange r("usr: clusters");
-        build_clusters(c, n, st);
-    }
-    mark(1, st);
-    cudaStream_t sd = c->side;
+    cudaStream_t sd = st;
     {
         NvtxRange r("usr: far chain (spread, convolutions, psi mean)");
         mark(3, sd);
         if (c->tc)
-            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, c->tc_bf16 ? 2 : 1, c->tcf.rho_hi,
+            usr::launch_spread(P.P, cluster_list(c), c->grid, c->tc_bf16 ? 2 : 1, c->tcf.rho_hi,
                                c->tcf.rho_lo, (c->vir || c->mlN > 0) ? c->d_rho32 : nullptr, c->d_spread_partial,
                                c->d_counters, c->d_mean, c->d_status, sd);
         else
-            usr::launch_spread(P.P, c->d_spos, c->d_cell_start, c->grid, 0, c->d_rho, nullptr, nullptr,
+            usr::launch_spread(P.P, cluster_list(c), c->grid, 0, c->d_rho, nullptr, nullptr,
                                c->d_spread_partial, c->d_counters, c->d_mean, c->d_status, sd);
+        {
+            NvtxRange rn("usr: near pairs");
+            mark(1, c->side);
+            usr::launch_near(c->max_groups, P.poly_deg, cluster_list(c), c->near, c->d_queue, c->d_nacc,
+                             c->vir ? c->d_vnear : nullptr, c->d_status, c->near_ctas_per_sm, c->side);
+            mark(2, c->side);
+            if (cudaEventRecord(c->ev_join, c->side) != cudaSuccess) return USR_ERR_CUDA;
+        }
         // the virial's grid products take FP32 rho without its mean; every other reader takes the mean off itself
         if (c->vir) usr::launch_sub_mean(c->G, c->tc ? c->d_rho32 : c->d_rho, c->d_rho32, c->d_mean, sd);
         mark(4, sd);
@@ -893,23 +882,16 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
             usr::launch_ml_prolong(c->ml, pc, t1, t2, c->d_psi, c->d_status, sd);
         }
         mark(8, sd);
-        usr::launch_gather(P.P, n, c->d_spos, c->d_psi, c->grid, c->d_far4, c->d_gather_partial, c->d_counters + 4,
+        usr::launch_gather(P.P, n, cluster_list(c), c->ncell, c->d_psi, c->grid, c->d_far4, c->d_gather_partial, c->d_counters + 4,
                            c->d_psi_mean, c->d_status, sd);
         mark(11, sd);
-        if (cudaEventRecord(c->ev_join, sd) != cudaSuccess) return USR_ERR_CUDA;
-    }
-    {
-        NvtxRange r("usr: near pairs");
-        usr::launch_near(c->max_groups, P.poly_deg, cluster_list(c), c->near, c->d_queue, c->d_nacc,
-                         c->vir ? c->d_vnear : nullptr, c->d_status, c->near_ctas_per_sm, st);
-        mark(2, st);
     }
     // join
     if (cudaStreamWaitEvent(st, c->ev_join, 0) != cudaSuccess) return USR_ERR_CUDA;
     mark(9, st);
     {
         NvtxRange r("usr: near + far, energy");
-        usr::launch_combine(n, c->d_spos, c->d_perm, c->d_nacc, c->d_far4, c->grid, out,
+        usr::launch_combine(n, cluster_list(c), c->ncell, c->d_nacc, c->d_far4, c->grid, out,
                             c->keep_parts ? c->d_near_dbg : nullptr, c->keep_parts ? c->d_far_dbg : nullptr,
                             c->d_gather_partial + usr::kGatherBlocks, c->d_counters + 1, en, c->d_netq,
                             c->d_status, st);
@@ -1116,7 +1098,10 @@ extern "C" usr_status usr_debug_cells(usr_ctx* c, int n, const float* xyzq, int*
     if (s != USR_OK) return s;
     if (n == 0) return USR_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    bin_and_cluster(c, n, (const float4*)xyzq, st);
+    usr::launch_bin_list(n, (const float4*)xyzq, c->boxf, c->ncell, c->d_count, c->d_cell_of, c->d_slot, c->d_wpos,
+                         c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, c->d_unsorted, c->d_status,
+                         st);
+    usr::launch_cell_sort(n, c->ncell, c->d_cell_start, c->d_unsorted, c->d_wpos, c->d_perm, c->d_spos, c->d_status, st);
     cudaMemcpyAsync(cell, c->d_cell_of, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(perm, c->d_perm, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(cell_start, c->d_cell_start, sizeof(int) * ((size_t)c->ncell + 1), cudaMemcpyDeviceToDevice, st);
@@ -1133,7 +1118,7 @@ extern "C" usr_status usr_debug_pairs(usr_ctx* c, int n, const float* xyzq, int*
     if (n == 0) return USR_OK;
     cudaStream_t st = (cudaStream_t)stream;
     bin_and_cluster(c, n, (const float4*)xyzq, st);
-    usr::launch_pairs(c->max_clusters, cluster_list(c), c->d_perm, c->near, count, (unsigned long long*)hash,
+    usr::launch_pairs(c->max_clusters, cluster_list(c), c->near, count, (unsigned long long*)hash,
                       c->d_status, st);
     return check_launch();
 }
@@ -1203,7 +1188,7 @@ extern "C" usr_status usr_stage_times(usr_ctx* c, float* ms)
     // (from, to) event pairs of the stages; the gather stage adds the multilevel coarse steps (if any) and
     // the far gather with psi's mean (11 - 7) to the combination (10 - 9); the wait for the later of the two
     // branches (between 2 or 11 and 9) is in no stage
-    static const int from[USR_NSTAGES] = {0, 1, 3, 4, 5, 6, 9}, to[USR_NSTAGES] = {1, 2, 4, 5, 6, 7, 10};
+    static const int from[USR_NSTAGES] = {0, 1, 3, 4, 5, 6, 9}, to[USR_NSTAGES] = {3, 2, 4, 5, 6, 7, 10};
     for (int k = 0; k < USR_NSTAGES; ++k) {
         float t = 0.f;
         if (cudaEventElapsedTime(&t, c->ev[from[k]], c->ev[to[k]]) != cudaSuccess) return USR_ERR_CUDA;

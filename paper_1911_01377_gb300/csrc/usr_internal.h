@@ -206,43 +206,38 @@ struct NearArgs {
     int max_clusters;     // clusters the cluster buffers hold
     int max_groups;       // groups the group table holds
     float rc2;            // (float)(r_c^2)
-    float two_over_rc2;   // 2 / r_c^2
     int n_explicit;
-    float ea[kMaxExplicit];
-    float einv[kMaxExplicit];
-    float el2[kMaxExplicit];   // -einv log2(e): exp(-u einv) = 2^(u el2)
-    float ne2[kMaxExplicit];   // -2 einv: factor of 2 dF/du
-    float poly[kMaxPolyDeg + 1];
-    // the same with their signs flipped, for the pair kernel's negated form of F (-F and its
-    // derivative accumulate with additions only)
-    float npoly[kMaxPolyDeg + 1];
-    float nea[kMaxExplicit];   // -ea
-    float nne2[kMaxExplicit];  // -ne2
-    float nd2fac;              // -2 * two_over_rc2: 2 dF/du from d(-F)/ds
+    // constants of the two-wide pair arithmetic, both halves equal: s = u * sfac - 1 with sfac = 2 / r_c^2;
+    // -F's polynomial in s and, as a polynomial of its own, the derivative 2 dF/du (degree one less); each
+    // explicit Gaussian exp(-u einv) = 2^(u el2), entering -F with nea and 2 dF/du with dea
+    float2 sfac;
+    float2 npoly[kMaxPolyDeg + 1];
+    float2 dpoly[kMaxPolyDeg];
+    float2 el2[kMaxExplicit], nea[kMaxExplicit], dea[kMaxExplicit];
 };
 
 /*
- * The cell list as the pair kernels read it: 8-slot clusters (paired layout,
- * see k_cluster_build) with their caller-sorted indices (-1 for padding rows),
+ * The cell list as the pair kernels read it: 8-slot clusters ((x, y, z, q)
+ * rows) with their caller indices (-1 for padding rows),
  * cells, bounding boxes, per-cell padded slot starts, and the groups of
  * consecutive clusters of one cell that one warp of the half-list kernel owns
- * (per-cell group starts, first cluster of each group).
+ * (per-cell group starts, descriptor of each group).
  */
 struct ClusterList {
     const float4* cpos;
-    const int* cidx;
+    const int* cperm;
     const int* ccell;
     const float4* bblo;
     const float4* bbhi;
     const int* pstart;
     const int* gfull;     // per cell: first full group (scan), total at [ncell]
     const int* gpart;     // per cell: its partial group's index after the full ones (scan), total at [ncell]
-    const int* gfirst;
+    const int4* gdesc;    // per group: (first cluster, cell, clusters, 0)
 };
 
 struct GridArgs {
     BoxF box;
-    int max_atoms;        // rows of the per-atom buffers (bounds of the debug build)
+    int max_slots;        // rows of the per-slot buffers (bounds of the debug build)
     float hh[3];          // h^2 / (2 sigma_s^2): exponent factor per stencil step
     float dfac[3];        // h / sigma_s^2: derivative factor
     float F0;             // self-interaction constant (per-atom potential)
@@ -277,7 +272,7 @@ struct ConvTcArgs {
     int n_out;              // output columns in all
     int nterms, nx, ny, nz;
     int stages;             // TMA ring depth
-    int tmem_cols;          // tensor-memory columns allocated (power of two >= 2 NT: two accumulators)
+    int tmem_cols;          // tensor-memory columns allocated (power of two >= NT, 2 NT in the TF32 form)
     int smem;               // dynamic shared memory per CTA (bytes; padded so that the CTAs an SM
                             // can hold never ask for more than 512 TMEM columns together)
     const float* mu;        // per-term mean of the 1D kernel (passes 1, 2)
@@ -321,15 +316,17 @@ void launch_ml_prolong(const MlArgs& m, const float* psi_c, float* t1, float* t2
 cudaError_t launch_bin(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
                        float4* wpos, int* cell_start, int* pstart, int* unsorted, int* perm, float4* spos,
                        int* status, cudaStream_t st);
-/* The sorted cell list (cell ids, counting sort, per-cell order by caller index); then the pair kernels'
-   clusters built from it (they may run on different streams, the second after the first). */
-void launch_bin_sorted(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
-                       float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue, int* unsorted,
-                       int* perm, float4* spos, int* status, cudaStream_t st);
+/* The cell list (cell ids, counting sort, any order within a cell); each cell in the order of caller indices (the
+   inspection entry points only); the 8-atom clusters. */
+void launch_bin_list(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
+                     float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue, int* unsorted,
+                     int* status, cudaStream_t st);
+void launch_cell_sort(int n, int ncell, const int* cell_start, const int* unsorted, const float4* wpos, int* perm,
+                      float4* spos, int* status, cudaStream_t st);
 void launch_clusters(int n, const BoxF& b, int ncell, const int* cell_start, const int* pstart, const int* gfull,
-                     const int* gpart, int* gfirst, const float4* spos, int* key, float4* cpos, int* cidx,
-                     int* ccell, float4* bblo, float4* bbhi, unsigned long long* near_acc, int max_clusters,
-                     int max_groups, int* status, cudaStream_t st);
+                     const int* gpart, int4* gdesc, const int* unsorted, const float4* wpos, int* key, float4* cpos,
+                     int* cperm, int* ccell, float4* bblo, float4* bbhi, unsigned long long* near_acc,
+                     int max_clusters, int max_groups, int* status, cudaStream_t st);
 /* Upper bound of the half-list kernel's groups for n atoms in ncell cells; clusters per group. */
 int near_max_groups(int n, int ncell);
 int near_group_clusters();
@@ -340,11 +337,11 @@ void launch_near(int max_groups, int deg, const ClusterList& L, const NearArgs& 
                  unsigned long long* acc, double* vir, int* status, int ctas_per_sm, cudaStream_t st);
 /* At most ctas_per_sm persistent pair-kernel CTAs per SM for this context (0: as many as fit). */
 void set_near_ctas_per_sm(usr_ctx* c, int ctas_per_sm);
-void launch_pairs(int max_clusters, const ClusterList& L, const int* perm, const NearArgs& a, int* count,
+void launch_pairs(int max_clusters, const ClusterList& L, const NearArgs& a, int* count,
                   unsigned long long* hash, int* status, cudaStream_t st);
 /* rho with its k = 0 mode still in it, as FP32 (split 0, rho) or a TF32 / BF16 operand split (1 / 2, rho and
    rho_lo, and an FP32 copy in rho32 when that is non-null), and its grid mean through spread_ctas(n) partial sums */
-void launch_spread(int P, const float4* spos, const int* cell_start, const GridArgs& g, int split, void* rho,
+void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, void* rho,
                    void* rho_lo, float* rho32, double* partial, unsigned int* counter, double* mean, int* status,
                    cudaStream_t st);
 int spread_ctas(const int* n);
@@ -363,16 +360,15 @@ usr_status make_tmap(CUtensorMap* m, const void* ptr, bool bf16, long long rows,
 size_t conv_tc_smem(const ConvTcArgs& g);
 usr_status conv_tc_setup(bool bf16, size_t smem);
 void launch_conv_tc(bool bf16, const ConvTcMaps& m, const ConvTcArgs& g, int batches, cudaStream_t st);
-/* far part at each of the n sorted atoms into far4 (-q grad phi, phi before the k = 0 correction), and psi's
-   grid mean into psi_mean through per-CTA sums in partial (kGatherBlocks CTAs at most) and the last CTA */
-void launch_gather(int P, int n, const float4* spos, const float* psi, const GridArgs& g, float4* far4,
+/* far part at each cluster slot that holds an atom into far4 (-q grad phi, phi before the k = 0 correction), and
+   psi's grid mean into psi_mean through per-CTA sums in partial (kGatherBlocks CTAs at most) and the last CTA */
+void launch_gather(int P, int n, const ClusterList& L, int ncell, const float* psi, const GridArgs& g, float4* far4,
                    double* partial, unsigned int* counter, double* psi_mean, int* status, cudaStream_t st);
 /* near + far in caller order into out (and the parts into near_dbg / far_dbg when non-null); energy[0..3] =
    total, near, far, self and *net_charge = sum q through per-CTA sums in partial (4 per CTA, kCombineBlocks
    CTAs at most) */
-void launch_combine(int n, const float4* spos, const int* perm, const unsigned long long* near_acc,
-                    const float4* far4, const GridArgs& g, float4* out, float4* near_dbg, float4* far_dbg,
-                    double* partial, unsigned int* counter, double* energy, double* net_charge, int* status,
-                    cudaStream_t st);
+void launch_combine(int n, const ClusterList& L, int ncell, const unsigned long long* near_acc, const float4* far4,
+                    const GridArgs& g, float4* out, float4* near_dbg, float4* far_dbg, double* partial,
+                    unsigned int* counter, double* energy, double* net_charge, int* status, cudaStream_t st);
 
 }  // namespace usr
