@@ -200,8 +200,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * 128;
-    const int batch = blockIdx.y, tile = blockIdx.z;
+    // the N tiles of an M tile side by side, so that they share its rows in L2
+    const int m0 = blockIdx.x / g.ntiles * 128;
+    const int batch = blockIdx.y, tile = blockIdx.x % g.ntiles;
     const int S = g.stages, NT = g.NT;
     const uint32_t a_bytes = 128 * kRowBytes;
     const uint32_t b_bytes = (uint32_t)NT * kRowBytes;
@@ -418,7 +419,7 @@ usr_status conv_tc_setup(bool bf16, size_t smem)
 
 void launch_conv_tc(bool bf16, const ConvTcMaps& m, const ConvTcArgs& g, int batches, cudaStream_t st)
 {
-    dim3 grid((g.lines + 127) / 128, batches, g.ntiles);
+    dim3 grid((g.lines + 127) / 128 * g.ntiles, batches);
     const size_t smem = (size_t)g.smem;
     if (bf16)
         launch_pdl(k_conv_tc<true>, grid, kTcThreads, smem, st, m.a_hi, m.a_lo, m.b_hi, m.b_lo, g);

@@ -34,9 +34,6 @@ struct NvtxRange {
 
 /* One tensor-core convolution (three passes): split operands (hi, lo), B tables and tensor maps per pass, the
    per-term means of the x and y kernels. */
-#ifndef USR_TC_MIN_CTAS
-#define USR_TC_MIN_CTAS 0     // split a tensor-core pass into more N tiles below this many CTAs
-#endif
 #ifndef USR_SIDE_PRIORITY
 #define USR_SIDE_PRIORITY 0   // priority of the far chain's stream: 0 highest, 1 default, 2 lowest
 #endif
@@ -200,16 +197,19 @@ void fill_box(const Plan& P, usr::BoxF& b)
 }
 
 /*
- * Tile shape of one tensor-core pass with n_out output columns and contraction K, over `ctas_m` M tiles (lines /
- * 128 x batches).  When that gives fewer than USR_TC_MIN_CTAS CTAs, the columns are split into more N tiles (16
- * columns at least) so that more SMs share the pass.
+ * N tiles of one tensor-core pass with n_out output columns (one more, the DC column, per tile).  At most 256
+ * columns to a tile.  TF32: at most 80, so that two CTAs fit an SM (two accumulators of 80 columns each take 256 of
+ * its 512 TMEM columns, a two-stage ring 106 KB of shared memory) and one's epilogue runs under the other's loads
+ * and MMAs; with one 144-column tile per CTA a 128^3 pass spent 13 us per CTA on loads, MMAs and epilogue in turn.
  */
-void tc_shape(usr::ConvTcArgs& a, int n_out, int K, bool bf16, long long ctas_m)
+int tc_tiles(int n_out, bool bf16) { return bf16 ? (n_out + 1 + 255) / 256 : (n_out + 78) / 79; }
+
+/* Tile shape of one tensor-core pass with n_out output columns and contraction K. */
+void tc_shape(usr::ConvTcArgs& a, int n_out, int K, bool bf16)
 {
     a.n_out = n_out;
     a.K = K;
-    a.ntiles = (n_out + 1 + 255) / 256;
-    while (ctas_m * a.ntiles < USR_TC_MIN_CTAS && (n_out + a.ntiles) / (a.ntiles + 1) >= 16) ++a.ntiles;
+    a.ntiles = tc_tiles(n_out, bf16);
     a.cols = (n_out + a.ntiles - 1) / a.ntiles;
     a.NT = ((a.cols + 1 + 15) / 16) * 16;
     a.tmem_cols = 32;
@@ -217,7 +217,7 @@ void tc_shape(usr::ConvTcArgs& a, int n_out, int K, bool bf16, long long ctas_m)
     const int kstage = bf16 ? 64 : 32;
     const int nk = (K + kstage - 1) / kstage;
     const size_t stage = (size_t)(2 * 128 + 2 * a.NT) * 128;
-    int S = (int)((200 * 1024) / stage);
+    int S = (int)((bf16 ? 200 * 1024 : 107 * 1024) / stage);
     S = std::min(S, std::min(nk, 4));
     a.stages = std::max(1, std::min(S, usr::kConvTcMaxStages));
     // keep (CTAs per SM) x (TMEM columns) <= 512 by padding the shared memory request: one CTA more than that must
@@ -296,7 +296,7 @@ double usr::plan_device_bytes(const Plan& P)
             b += 4 * Gc * 2 * (1 + 2 * Nc) + 8 * Nc + 4 * Gc;
             const double n_out[3] = {cx, cy, cz}, K[3] = {cx, cy, Nc * cz}, bat[3] = {Nc, Nc, 1};
             for (int p = 0; p < 3; ++p) {
-                const double nt = std::floor((n_out[p] + 1 + 255) / 256);
+                const double nt = tc_tiles((int)n_out[p], false);
                 const double cols = std::ceil(n_out[p] / nt);
                 const double NT = std::ceil((cols + 1) / 16) * 16;
                 b += 2 * 4 * bat[p] * nt * NT * K[p];
@@ -313,7 +313,7 @@ double usr::plan_device_bytes(const Plan& P)
         b += es * G * 2 * (1 + 2 * N) + 8 * N;
         const double n_out[3] = {nx, ny, nz}, K[3] = {nx, ny, N * nz}, bat[3] = {N, N, 1};
         for (int p = 0; p < 3; ++p) {
-            const double nt = std::floor((n_out[p] + 1 + 255) / 256);
+            const double nt = tc_tiles((int)n_out[p], P.p.conv == USR_CONV_BF16X3);
             const double cols = std::ceil(n_out[p] / nt);
             const double NT = std::ceil((cols + 1) / 16) * 16;
             b += 2 * es * bat[p] * nt * NT * K[p];
@@ -347,7 +347,7 @@ usr_status setup_tc(usr_ctx* c, TcConv& t, bool bf, int N, int nx, int ny, int n
     for (int ps = 0; ps < 3; ++ps) {
         usr::ConvTcArgs& a = t.targs[ps];
         std::memset(&a, 0, sizeof(a));
-        tc_shape(a, n_out[ps], Ks[ps], bf, (long long)((lines[ps] + 127) / 128) * batches[ps]);
+        tc_shape(a, n_out[ps], Ks[ps], bf);
         const size_t nB = (size_t)batches[ps] * a.ntiles * a.NT * a.K;
         if ((s = ensure(c, &t.Bt_hi[ps], es * nB)) != USR_OK || (s = ensure(c, &t.Bt_lo[ps], es * nB)) != USR_OK)
             return s;
