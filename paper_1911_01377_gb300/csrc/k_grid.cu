@@ -140,22 +140,33 @@ void launch_grid_dot(const GridArgs& g, const float* a, const float* b, double s
 }
 
 /*
- * W = W_near + delta E_far + 1/2 <rho, psi_ab>: near from the pair kernel's per-unit slots (in unit
- * order; the unit count follows from the group totals of the cell list), far from the six grid dot
- * products (already halved) and E_far.
+ * W = W_near + delta E_far + 1/2 <rho, psi_ab>: near from the pair kernel's per-unit slots (the unit count
+ * follows from the group totals of the cell list; every thread sums its units in order, then the threads in a
+ * fixed tree), far from the six grid dot products (already halved) and E_far.
  */
-__global__ void k_virial_finalize(const double* __restrict__ near_w, ClusterList L, int ncell, int nsplit,
-                                  const double* __restrict__ dots, const double* __restrict__ energy,
-                                  double* __restrict__ W)
+__global__ void __launch_bounds__(1024) k_virial_finalize(const double* __restrict__ near_w, ClusterList L, int ncell,
+                                                          int nsplit, const double* __restrict__ dots,
+                                                          const double* __restrict__ energy, double* __restrict__ W)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double red[32][6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int units = nsplit * (L.gfull[ncell] + L.gpart[ncell]);
     double wn[6] = {0, 0, 0, 0, 0, 0};
-    for (int w = 0; w < units; ++w)
-        for (int c = 0; c < 6; ++c) wn[c] += near_w[6 * w + c];
+    for (int w = threadIdx.x; w < units; w += 1024)
+        for (int c = 0; c < 6; ++c) wn[c] += near_w[6 * (size_t)w + c];
+    for (int c = 0; c < 6; ++c) {
+        const double v = warp_sum_d(wn[c]);
+        if (lane == 0) red[warp][c] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     const double ef = energy[2];
     double t[6];
-    for (int c = 0; c < 6; ++c) t[c] = wn[c] + dots[c] + (c < 3 ? ef : 0.0);
+    for (int c = 0; c < 6; ++c) {
+        double v = 0.0;
+        for (int w = 0; w < 32; ++w) v += red[w][c];
+        t[c] = v + dots[c] + (c < 3 ? ef : 0.0);
+    }
     const int map[9] = {0, 3, 4, 3, 1, 5, 4, 5, 2};
     for (int e = 0; e < 9; ++e) W[e] = t[map[e]];
 }
@@ -163,7 +174,7 @@ __global__ void k_virial_finalize(const double* __restrict__ near_w, ClusterList
 void launch_virial_finalize(const double* near_w, const ClusterList& L, int ncell, const double* dots,
                             const double* energy, double* W, cudaStream_t st)
 {
-    k_virial_finalize<<<1, 32, 0, st>>>(near_w, L, ncell, near_splits(), dots, energy, W);
+    k_virial_finalize<<<1, 1024, 0, st>>>(near_w, L, ncell, near_splits(), dots, energy, W);
 }
 
 /* ------------------------------------------------------------------ gather */
@@ -199,6 +210,40 @@ __host__ __device__ constexpr int gather_lanes(int P)
     return USR_GATHER_LANES ? USR_GATHER_LANES : (P == 10 ? 5 : 4);
 }
 
+/* The CTAs' shares of psi's grid sum in a fixed order (the last CTA), then its mean. */
+__device__ __forceinline__ void finish_psi_mean(CSum ps, long long G, double* __restrict__ partial,
+                                                unsigned int* __restrict__ counter, double* __restrict__ psi_mean)
+{
+    __shared__ double red[kGWarps];
+    __shared__ int is_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double t = warp_sum_c(ps);
+    if (lane == 0) red[warp] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < kGWarps; ++w) v += red[w];
+        partial[blockIdx.x] = v;
+        __threadfence();
+        is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    double a = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += kGThreads) a += ((volatile double*)partial)[k];
+    a = warp_sum_d(a);
+    __syncthreads();
+    if (lane == 0) red[warp] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < kGWarps; ++w) v += red[w];
+        *psi_mean = v / (double)G;
+        *counter = 0u;
+    }
+}
+
 template <int P>
 __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 256 / kGThreads)
     k_gather(const float4* __restrict__ cpos, const int* __restrict__ nslots, const float* __restrict__ psi, GridArgs g,
@@ -211,8 +256,6 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
     constexpr int NC = (P + LPA - 1) / LPA;    // stencil columns per lane
     constexpr int APW = 32 / LPA;              // atoms per warp pass
     constexpr int APC = kGWarps * APW;         // atoms per CTA pass
-    __shared__ double red[kGWarps];
-    __shared__ int is_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slot = lane / LPA, u = lane % LPA;
     const int n0 = g.box.n[0], n1 = g.box.n[1], n2 = g.box.n[2];
@@ -314,32 +357,156 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
             far4[s] = make_float4(-qi * ax, -qi * ay, -qi * az, aphi);
         }
     }
-    // psi's grid sum over all CTAs in a fixed order (the last CTA), then its mean
-    const double t = warp_sum_c(ps);
-    if (lane == 0) red[warp] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < kGWarps; ++w) v += red[w];
-        partial[blockIdx.x] = v;
-        __threadfence();
-        is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    finish_psi_mean(ps, G, partial, counter, psi_mean);
+}
+
+/*
+ * The gather of the wide stencils (12 points and more) on an even x extent: one warp per atom.  A lane holds two
+ * neighbouring x points, aligned (the stencil's points plus zero weights at its ends: NP lanes cover a row), of the
+ * rows y = r, r + R, ... (R = 32 / NP rows side by side); it contracts z first, all of a lane's loads
+ * independent, then its x points and rows; the warp sums the lanes at the end.  The z weights come from
+ * shared memory (lane k evaluates weight k), the x and y weights are the lane's own.
+ *
+ * Bound: L1 wavefronts (the rows of a load fall on overlapping banks).  A row is one two-wide load where k_gather
+ * spreads each load over 8 atoms' rows: alone on the slab (12 points) 90 -> 76 us.  With 10 points the two are
+ * equal (130 against 124 us for 200 k charges) and with 8, four points to a lane, this form is slower (44 against
+ * 35 us on the slab): the weights then cost more than the rows.
+ */
+template <int P, int V>
+struct GatherShape {
+    static constexpr int NP = (P + 2 * (V - 1)) / V;              // lanes per row: P points at any offset mod V
+    static constexpr int R = 32 / NP < P ? 32 / NP : P;           // rows side by side
+    static constexpr int BL = (P + R - 1) / R;                    // rows per lane
+};
+
+template <int V>
+struct VecOf;
+template <>
+struct VecOf<1> { typedef float T; };
+template <>
+struct VecOf<2> { typedef float2 T; };
+template <>
+struct VecOf<4> { typedef float4 T; };
+
+template <int P, int V>
+__global__ void __launch_bounds__(kGThreads, 8)
+    k_gather_wide(const float4* __restrict__ cpos, const int* __restrict__ nslots, int per, const float* __restrict__ psi, GridArgs g,
+             float4* __restrict__ far4, double* __restrict__ partial, unsigned int* __restrict__ counter,
+             double* __restrict__ psi_mean, int* __restrict__ status)
+{
+    pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
+    constexpr int H = P / 2;
+    typedef GatherShape<P, V> Sh;
+    typedef typename VecOf<V>::T Vec;
+    __shared__ float2 zw[kGWarps][P];          // z weight and its derivative factor
+    __shared__ unsigned int zo[kGWarps][P];    // offset of the plane
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n0 = g.box.n[0], n1 = g.box.n[1], n2 = g.box.n[2];
+    const unsigned int plane = (unsigned int)n0 * n1;
+    // psi's mean (its rounding-level k = 0 mode): this CTA's share of the grid sum first
+    CSum ps;
+    const long long G = (long long)plane * n2;
+    for (long long i = (long long)blockIdx.x * kGThreads + threadIdx.x; i < G; i += (long long)gridDim.x * kGThreads)
+        ps.add(psi[i]);
+    const int slot = lane % Sh::NP, row = lane / Sh::NP;
+    const int ns = *nslots;
+    for (int c0 = blockIdx.x * (kGWarps * per); c0 < ns; c0 += gridDim.x * (kGWarps * per)) {
+        const int s1 = min(ns, c0 + kGWarps * per);
+        for (int s = c0 + warp; s < s1; s += kGWarps) {
+            const float4 p = cpos[s];
+            if (p.x < -5.0e5f) continue;           // a padding slot (near -1e6)
+            const float ux = p.x * g.box.gs[0], uy = p.y * g.box.gs[1], uz = p.z * g.box.gs[2];
+            const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
+            const int b0 = (int)fx - H + 1, b1 = (int)fy - H + 1, b2 = (int)fz - H + 1;
+            const float tx = grid_frac(g.box, 0, p.x, fx), ty = grid_frac(g.box, 1, p.y, fy);
+            if (lane < P) {
+                const float d = (float)(lane - H + 1) - grid_frac(g.box, 2, p.z, fz);
+                const float w = __expf(-d * d * g.hh[2]);
+                zw[warp][lane] = make_float2(w, w * d * g.dfac[2]);
+                zo[warp][lane] = (unsigned int)wrap_once(b2 + lane, n2) * plane;
+            }
+            // this lane's x points (weight 0 outside the stencil and for lanes past the last row)
+            const int xs = (b0 & ~(V - 1)) + V * slot;
+            float wx[V], dx[V];
+            #pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int k = xs + v - b0;
+                const float d = (float)(k - H + 1) - tx;
+                wx[v] = k >= 0 && k < P && row < Sh::R ? __expf(-d * d * g.hh[0]) : 0.f;
+                dx[v] = wx[v] * d * g.dfac[0];
+            }
+            const unsigned int xo = (unsigned int)wrap_once(xs, n0);
+            unsigned int off[Sh::BL];
+            float wy[Sh::BL], dy[Sh::BL];
+            #pragma unroll
+            for (int b = 0; b < Sh::BL; ++b) {
+                const int j = row + Sh::R * b;
+                const float d = (float)(j - H + 1) - ty;
+                wy[b] = j < P ? __expf(-d * d * g.hh[1]) : 0.f;
+                dy[b] = wy[b] * d * g.dfac[1];
+                off[b] = (unsigned int)wrap_once(b1 + (j < P ? j : 0), n1) * (unsigned int)n0 + xo;
+            }
+            __syncwarp();
+            float c0v[Sh::BL][V], c1v[Sh::BL][V];
+            #pragma unroll
+            for (int b = 0; b < Sh::BL; ++b)
+                #pragma unroll
+                for (int v = 0; v < V; ++v) c0v[b][v] = c1v[b][v] = 0.f;
+            #pragma unroll
+            for (int k = 0; k < P; ++k) {
+                const float2 w = zw[warp][k];
+                const unsigned int z = zo[warp][k];
+                #pragma unroll
+                for (int b = 0; b < Sh::BL; ++b) {
+                    const Vec q = __ldg(reinterpret_cast<const Vec*>(psi + (z + off[b])));
+                    const float* f = reinterpret_cast<const float*>(&q);
+                    if (V == 1) {
+                        c0v[b][0] = fmaf(w.x, f[0], c0v[b][0]);
+                        c1v[b][0] = fmaf(w.y, f[0], c1v[b][0]);
+                    } else {
+                        #pragma unroll
+                        for (int v = 0; v + 1 < V; v += 2) {
+                            const float2 f2 = make_float2(f[v], f[v + 1]);
+                            const float2 r0 = __ffma2_rn(make_float2(w.x, w.x), f2, make_float2(c0v[b][v], c0v[b][v + 1]));
+                            const float2 r1 = __ffma2_rn(make_float2(w.y, w.y), f2, make_float2(c1v[b][v], c1v[b][v + 1]));
+                            c0v[b][v] = r0.x;
+                            c0v[b][v + 1] = r0.y;
+                            c1v[b][v] = r1.x;
+                            c1v[b][v + 1] = r1.y;
+                        }
+                    }
+                }
+            }
+            float aphi = 0.f, ax = 0.f, ay = 0.f, az = 0.f;
+            #pragma unroll
+            for (int b = 0; b < Sh::BL; ++b) {
+                float r0 = 0.f, r1 = 0.f, r2 = 0.f;
+                #pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    r0 = fmaf(wx[v], c0v[b][v], r0);
+                    r1 = fmaf(dx[v], c0v[b][v], r1);
+                    r2 = fmaf(wx[v], c1v[b][v], r2);
+                }
+                aphi = fmaf(wy[b], r0, aphi);
+                ax = fmaf(wy[b], r1, ax);
+                ay = fmaf(dy[b], r0, ay);
+                az = fmaf(wy[b], r2, az);
+            }
+            // reduce-scatter over the warp: lane 8 c ends with component c of (x, y, z, phi)
+            const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0;
+            const float t0 = __shfl_xor_sync(0xffffffffu, h4 ? ax : az, 16);
+            const float t1 = __shfl_xor_sync(0xffffffffu, h4 ? ay : aphi, 16);
+            const float k0 = (h4 ? az : ax) + t0, k1 = (h4 ? aphi : ay) + t1;
+            const float t2 = __shfl_xor_sync(0xffffffffu, h3 ? k0 : k1, 8);
+            float v = (h3 ? k1 : k0) + t2;
+            #pragma unroll
+            for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if ((lane & 7) == 0 && USR_IN_BOUNDS(s, g.max_slots, status))
+                reinterpret_cast<float*>(far4 + s)[lane >> 3] = lane < 24 ? -p.w * v : v;
+            __syncwarp();   // zw and zo are rewritten
+        }
     }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    double a = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += kGThreads) a += ((volatile double*)partial)[k];
-    a = warp_sum_d(a);
-    __syncthreads();
-    if (lane == 0) red[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < kGWarps; ++w) v += red[w];
-        *psi_mean = v / (double)G;
-        *counter = 0u;
-    }
+    finish_psi_mean(ps, G, partial, counter, psi_mean);
 }
 
 /*
@@ -438,10 +605,27 @@ static int gather_blocks(int n, int P)
     return std::max(1, std::min(kGatherBlocks, (n + apc - 1) / apc));
 }
 
+template <int P>
+static void gather_wide(int n, const ClusterList& L, int ncell, const float* psi, const GridArgs& g, float4* far4,
+                        double* partial, unsigned int* counter, double* psi_mean, int* status, cudaStream_t st)
+{
+    // slots per warp and pass: up to 8 neighbours (their rows overlap in L1), fewer when that would leave warps idle
+    const int slots = max_slots_of(n, ncell), per = std::max(1, std::min(8, slots / (kGWarps * kGatherBlocks)));
+    const int nb = std::max(1, std::min(kGatherBlocks, (slots + kGWarps * per - 1) / (kGWarps * per)));
+    launch_with(-1, k_gather_wide<P, 2>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, per, psi, g, far4, partial,
+                counter, psi_mean, status);
+}
+
 void launch_gather(int P, int n, const ClusterList& L, int ncell, const float* psi, const GridArgs& g, float4* far4,
                    double* partial, unsigned int* counter, double* psi_mean, int* status, cudaStream_t st)
 {
     const int nb = gather_blocks(max_slots_of(n, ncell), P);
+    if (P >= 12 && g.box.n[0] % 2 == 0) {
+        if (P == 12) gather_wide<12>(n, L, ncell, psi, g, far4, partial, counter, psi_mean, status, st);
+        else if (P == 14) gather_wide<14>(n, L, ncell, psi, g, far4, partial, counter, psi_mean, status, st);
+        else gather_wide<16>(n, L, ncell, psi, g, far4, partial, counter, psi_mean, status, st);
+        return;
+    }
     switch (P) {
         USR_GATHER_CASE(8)
         USR_GATHER_CASE(10)
