@@ -46,9 +46,9 @@ METRIC = "u-series E+F atom-evals/s at rms rel force err ≤1e-4; serving p50/p9
 UNIT = "atom-evals/s"
 WORKLOAD = "membrane_slab"
 SWEEP = (8.0, 9.0, 10.0, 11.0, 12.0, 13.0)
-# kernels of one evaluation: bin_count, scan, place, cell_build, near, spread, tile_reduce, conv x, conv y,
-# conv z, grid_mean, gather
-KERNELS_PER_EVAL = 12
+# kernels of one evaluation: bin_count, scan, place, cluster_build, near, spread, conv x, conv y, conv z, gather,
+# combine
+KERNELS_PER_EVAL = 11
 FP32_PEAK_DERIVED_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12   # SMs x FP32 lanes x 2 (FMA) x max SM clock
 # algorithmic flops of one unordered pair inside r_c, the unit of the pair kernel's roofline: the midpoint of
 # 30-50 flops for the arithmetic any pair kernel of Eq. 20 needs (the displacement and r^2, 1/r, F(r) and its
@@ -57,7 +57,7 @@ NEAR_FLOPS_PER_PAIR = 40
 # DRAM bytes (read + write) per launch of the pair kernel over this sweep, averaged over its six launches (one
 # per cutoff) in one ncu capture of `bench.py --steps 1 --warmup 3 --serve-systems 0 --no-scale`; None whenever
 # the pair kernel has changed since that capture
-NEAR_TRAFFIC_BYTES = 3.718e6
+NEAR_TRAFFIC_BYTES = None
 # forms: (name, conv, spread_points, spread_sigma_over_h)
 CHOSEN = ("bf16x3_gse8", 2, 8, 0.83)
 COMPARATORS = (("fp32_gse8", 0, 8, 0.83), ("fp32_tight12", 0, 12, 1.0))

@@ -198,12 +198,12 @@ usr_status usr_info(const usr_ctx* ctx, usr_plan_info* out);
  *          phi_i = dE/dq_i (the potential at i with i's self term included)
  *   energy device, 4 doubles: E, E_near, E_far, E_self (may be NULL)
  * n = 0 writes zero energies.  USR_ERR_CAPACITY if n > max_atoms.
- * Internally the far part runs on a second stream of the context, forked from
- * `stream` after the cell list and joined back before the near + far
- * combination, so the call stays ordered on `stream` (and capturable) as one
- * unit.  A context's buffers are reused by every call: calls on one context
- * from different streams must be ordered by the caller (an event between
- * them).  Cost: the cell list orders each cell by counting, quadratic in the
+ * Internally the pair kernel of the near part runs on a second stream of the
+ * context, forked from `stream` after the cell list and joined back before the
+ * near + far combination, while the far part runs on `stream`, so the call
+ * stays ordered on `stream` (and capturable) as one unit.  A context's
+ * buffers are reused by every call: calls on one context from different
+ * streams must be ordered by the caller (an event between them).  Cost: the cell list orders each cell by counting, quadratic in the
  * cell's occupancy, and the near part grows with the pairs inside r_c; at the
  * densities the method is made for (about 0.1 charges per cubic Angstrom)
  * cells hold tens to a few hundred atoms, while charges piled into one cell
@@ -420,8 +420,8 @@ usr_status usr_set_profiling(usr_ctx* ctx, int on);
  * ms must hold USR_NSTAGES floats; with profiling level 2 only the near stage
  * (index 1) is measured and the others read 0.  The far chain (spread,
  * conv_x/y/z, then the multilevel coarse steps and the far gather, both
- * counted in gather) runs on the context's own high-priority stream,
- * concurrently with the near stage on the caller's stream; gather also counts
+ * counted in gather) runs on the caller's stream, concurrently with the near
+ * stage on the context's own stream; gather also counts
  * the near + far combination after the two streams join.  So the stages can
  * add up to more than the evaluation's duration.
  */

@@ -28,6 +28,17 @@
  * atomics), and the sum is exact.  Each part is an FP32 sum formed in a fixed
  * order, rounded once to the fixed-point grid.
  *
+ * The i atoms of a group, its boxes and a unit's neighbour cells lie in the warp's shared memory; the unit's
+ * candidates (all its cells together) are tested 32 at a time, the next surviving j-cluster's atoms are loaded
+ * while the current one's steps run, and the next unit is taken from the queue during the current one.
+ *
+ * Bound: issue slots and the latency of the step's chain (55 % of the slots used at 16 warps per SM; about 105
+ * instructions per step that has a pair inside r_c, 32 of them two-wide FP32).  Alone, slab at r_c = 8 / 10 / 13 A:
+ * 76 / 98 / 179 us, 200 k charges at 9 A 246 us, 1.06 M at 10 A 1.44 ms, against 92 / 126 / 212 us, 305 us and 1.75
+ * ms with i atoms in registers, clusters in Morton order and one scan per neighbour cell.  Not kept: constants
+ * pinned in registers (no change: the instructions take them from constant memory); the surviving clusters as a
+ * list in shared memory (the loop is no longer uniform: 110 us at 10 A); 3, 5, 6, 7 or 8 CTAs per SM.
+ *
  * Per pair: r^2 by the single-precision predicate on d = x_i - (x_j + shift);
  * 1/r by rsqrt; F(u = r^2) = explicit narrow Gaussians plus a polynomial in
  * s = 2u / r_c^2 - 1 (Horner, value and derivative).
@@ -44,8 +55,8 @@
 #define USR_NEAR_GI 4
 #endif
 #ifndef USR_NEAR_MINB
-#define USR_NEAR_MINB 5     // CTAs of 128 threads per SM the register budget is set for (96 registers:
-                            // 20 warps per SM, 122 us at r_c = 10 A on the slab against 133 us with 16)
+#define USR_NEAR_MINB 5     // CTAs of 128 threads per SM the register budget is set for (90 registers used; 4
+                            // CTAs then leave 16 k registers of an SM to the far chain)
 #endif
 
 namespace usr {
@@ -533,9 +544,6 @@ __global__ void __launch_bounds__(128) k_pairs_count(ClusterList L, NearArgs a,
 /* ------------------------------------------------------------ launchers */
 
 constexpr int kNearGroup = USR_NEAR_GI;
-#ifndef USR_NEAR_RESERVE
-#define USR_NEAR_RESERVE 0
-#endif
 
 int near_max_groups(int n, int ncell) { return (int)(((long long)n + (8LL * kNearGroup - 1) * ncell) / (8 * kNearGroup)) + 1; }
 
@@ -560,16 +568,12 @@ static int2 persistent_shape(K kernel)
 }
 
 /*
- * Grid of the persistent pair kernel: the CTAs the SMs hold at once, less USR_NEAR_RESERVE per SM
- * (slots left for the far-part kernels of the second stream), or at most ctas_per_sm per SM when that
- * is given (the serving loop runs several systems at once); at least one per SM.  Measured on the
- * membrane slab, the pair kernel with every slot (reserve 0) gives the shortest evaluation: it runs
- * 13% faster than with one slot per SM left free, and the far chain, latency-bound, gains less from
- * running beside it than the pair kernel loses.
+ * Grid of the persistent pair kernel: the CTAs the SMs hold at once, or at most ctas_per_sm per SM when that
+ * is given (an evaluation leaves one slot per SM to the far chain beside it); at least one per SM.
  */
 static int persistent_grid(int2 shape, int ctas_per_sm, int units_max)
 {
-    int per_sm = shape.x - USR_NEAR_RESERVE;
+    int per_sm = shape.x;
     if (ctas_per_sm > 0) per_sm = std::min(per_sm, ctas_per_sm);
     if (per_sm < 1) per_sm = 1;
     return std::max(1, std::min(per_sm * shape.y, (units_max + 3) / 4));

@@ -3,10 +3,10 @@
  * creation (plan + device allocation + table upload), the evaluation
  * sequence on one stream, host-buffer evaluation, status and inspection.
  *
- * Evaluation sequence (one stream, no host synchronisation, no allocation):
- *   bin + sort (cell list) -> near pair kernel (Eq. 20) -> spread ->
- *   x / y / z convolution passes (Sec. V, Eqs. 31-32) -> gather + combine +
- *   FP64 energy reduction.
+ * Evaluation sequence (no host synchronisation, no allocation):
+ *   cell list and clusters -> { pair kernel (Eq. 20) on a stream forked off |
+ *   spread -> x / y / z convolution passes (Sec. V, Eqs. 31-32) -> gather }
+ *   -> combine with the FP64 energy reduction.
  */
 #include <algorithm>
 #include <cstdio>
@@ -34,11 +34,9 @@ struct NvtxRange {
 
 /* One tensor-core convolution (three passes): split operands (hi, lo), B tables and tensor maps per pass, the
    per-term means of the x and y kernels. */
-#ifndef USR_SIDE_PRIORITY
-#define USR_SIDE_PRIORITY 0   // priority of the far chain's stream: 0 highest, 1 default, 2 lowest
-#endif
 #ifndef USR_NEAR_CTAS
-#define USR_NEAR_CTAS 4   // one CTA slot per SM left to the far chain (measured: 5 and 3 slower)
+#define USR_NEAR_CTAS 4   // one CTA slot per SM left to the far chain (evaluations with 3 / 4 / 5 CTAs: slab r_c = 13 A
+                          // 286 / 257 / 262 us, tight 315 / 299 / 304, 1.06 M charges 2.33 / 2.24 / 2.32 ms)
 #endif
 
 struct TcConv {
@@ -971,11 +969,8 @@ usr_status init_ctx(usr_ctx* c, const usr_params* p)
     for (auto& e : c->ev) cudaEventCreate(&e);
     c->ev_made = true;
     {
-        int least = 0, greatest = 0;
-        if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking,
-                                         USR_SIDE_PRIORITY == 0 ? greatest : (USR_SIDE_PRIORITY == 1 ? 0 : least))
-                != cudaSuccess ||
+        // default priority: above it, the same times within 0.3 us up to 200 k charges and 2.232 ms against 2.223 at 1.06 M
+        if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)
             return USR_ERR_CUDA;
