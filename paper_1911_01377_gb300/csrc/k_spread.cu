@@ -22,12 +22,14 @@
  *
  * Bound: issue slots (about 45 % of them used) and the latency of the list.  (P + 15) / 16 ((P + 7) / 8)^2
  * bricks per atom at about 25 instructions each, and one to two per atom listed.  Alone (ncu): 42 us on the
- * slab at r_c = 8 A (P = 8), 122 us for 200 k charges (P = 10).  The earlier form (shared-memory tiles per
+ * slab at r_c = 8 A (P = 8), 111 us for 200 k charges (P = 10).  The earlier form (shared-memory tiles per
  * block of cells, one read-modify-write per stencil point, then a reduction over overlapping tiles) took
  * 36 + 23 us and 157 + 73 us: 940 instructions per atom at P = 10 against 290, held by shared-memory
  * wavefronts and by the tiles' 13-fold halo traffic.  Bricks summed by FP32 FMAs instead took 217 us (the
  * register side of broadcast loads), this contraction with weight rows shared by a CTA's warps 172 us
- * (barriers).
+ * (barriers).  Not kept either: the sums by two-wide FP32 FMAs of each warp (evaluations 1 to 3 % slower, the
+ * FP32 pipe is the pair kernel's); up to 16 warps per brick on one flattened list (68 -> 65 us per evaluation of
+ * 2 k charges, 598 -> 606 us of 200 k).
  */
 #include <algorithm>
 

@@ -406,8 +406,8 @@ usr_status make_plan(const usr_params* pp, Plan* out)
             ++P.n_explicit;
         }
     }
-    // cell blocks of the spreading / interpolation kernels: cores of about 16
-    // grid points (the tiles' halo of P + 3 points makes small cores costly),
+    // geometry of blocks of cells with their stencils' halo.  No kernel stages such tiles any more; the plan keeps
+    // them because they decide which parameters are accepted: cores of about 16 grid points,
     // tiles within kTileMaxSmem, at least 304 blocks (two per SM) when the cell list allows,
     // at most 64 (z, y) cell rows per block
     {
