@@ -6,12 +6,23 @@
  * the convolutions takes it off its row sums).
  *
  * Owner-computes, as a contraction over atoms: a warp owns a brick of 16 x 8 x 8 grid points (x, y, z) and
- * for eight atoms at a time adds the rank-8 product X YZ_z of their x weights (16 points x 8 atoms, charge
- * included) and their y weights times the z weight of plane z (8 atoms x 8 points) for each of its 8 planes,
- * on the tensor cores (mma.sync m16n8k8) with the sums in registers.  The operands are split into TF32 high
- * and low parts (to nearest) and three products are accumulated in FP32, which keeps about 22 bits of each
- * factor.  The tcgen05 form would need the y-z
- * products in shared memory, 256 bytes per atom and plane; here they are formed in registers.
+ * for eight atoms at a time adds the product X YZ_z of their x weights (16 points x 8 atoms, charge included)
+ * and their y weights times the z weight of plane z (8 atoms x 8 points) for each of its 8 planes, with the
+ * brick's sums in registers.  Two forms:
+ *
+ *   split forms (TF32x3 and BF16x3 convolutions)  on the tensor cores (mma.sync m16n8k8).  The operands are
+ *       split into TF32 high and low parts (to nearest) and three products are accumulated in FP32, which keeps
+ *       about 22 bits of each factor; the MMA truncates its sums, so a brick's sums carry a bias of about 1e-7.
+ *       The tcgen05 form would need the y-z products in shared memory, 256 bytes per atom and plane; here they
+ *       are formed in registers.
+ *   F32 (FP32 convolutions)  two-wide FP32 FMAs, a lane four x points of one y in every plane, in blocks of 16
+ *       atoms that are summed apart (a point of a 12-point stencil receives about 170 terms).  The bias of the
+ *       tensor-core form does not cancel over the net charge of a region: with it, the far potential of a drop
+ *       of water in vacuum (6,000 charges in 90 A) was off by 6.2e-6 of its norm, with FMAs in one chain by
+ *       4.6e-6, with blocks by 1.8e-6 (1.0e-6 is the method's own error).  Evaluations in the FP32 form with
+ *       FMAs / on the tensor cores: 3,000 charges 70.3 / 71.0 us, 7,013 ions 90.9 / 92.7, slab 272 / 269.
+ *       Up to 249 bricks eight warps share one and an SM gets at most two CTAs, so their registers are not capped
+ *       at 128 (they would spill 108 bytes: 3,000 charges 71.8 us).
  *
  * Every warp works by itself: it lists the atoms of the cells its brick's stencils can reach (rows of cells,
  * periodic images as separate rows), keeps those that do reach in a small queue in list order, and evaluates
@@ -104,9 +115,17 @@ struct SpreadWarp {
     float z[8][kBrick];      // z weights of the current eight atoms
 };
 
-template <int S, int WARPS>
+/* The FP32 form's further weights of the current eight atoms (rows of x weights 24 floats apart: a warp's stores of
+   four rows then touch each bank once). */
+struct SpreadWeights {
+    float x[8][kBrickX + 8];
+    float y[8][kBrick];
+};
+
+template <int S, int WARPS, bool F32>
 struct SpreadShared {
     SpreadWarp w[WARPS];
+    SpreadWeights xy[F32 ? WARPS : 1];
     float4 share[S > 1 ? (WARPS - WARPS / S) * 256 : 1];   // bricks' shares of the splits after the first
     double red[WARPS];
     int is_last;
@@ -116,8 +135,8 @@ struct SpreadShared {
 
 /* out: 0 FP32 rho; 1 and 2 the operand split of the tensor-core convolutions, rho = hi + lo with hi rounded to
    TF32 (1) or BF16 (2).  rho32: FP32 copy beside a split (may be null). */
-template <int S, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4* __restrict__ pos,
+template <int S, int WARPS, bool F32>
+__global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) k_spread(const float4* __restrict__ pos,
                                                         const int* __restrict__ pstart, GridArgs g, int P,
                                                         int bricks_x, int bricks_y, int bricks, int out,
                                                         void* __restrict__ rho, void* __restrict__ rho_lo,
@@ -127,7 +146,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
     constexpr int NB = WARPS / S;
-    __shared__ __align__(16) SpreadShared<S, WARPS> sh;
+    __shared__ __align__(16) SpreadShared<S, WARPS, F32> sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = P / 2;
     const int n0 = g.box.n[0], n1 = g.box.n[1], n2 = g.box.n[2];
@@ -143,11 +162,17 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
     // exp(-d^2 hh) = 2^(d^2 c)
     const float kl = -1.4426950408889634f;
     const float cx = g.hh[0] * kl, cy = g.hh[1] * kl, cz = g.hh[2] * kl;
-    float acc[8][4];         // per plane z: (x, y) = (gq, 2 tq), (gq, 2 tq + 1), (gq + 8, 2 tq), (gq + 8, 2 tq + 1)
+    // per plane z, the points (x, y): (gq, 2 tq), (gq, 2 tq + 1), (gq + 8, 2 tq), (gq + 8, 2 tq + 1); F32: (4 tq, gq)
+    // .. (4 tq + 3, gq), acc holds the atoms since the last fold into sum
+    float acc[8][4], sum[F32 ? 8 : 1][4];
+    int groups = 0;
     #pragma unroll
     for (int z = 0; z < 8; ++z)
         #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[z][k] = 0.f;
+        for (int k = 0; k < 4; ++k) {
+            acc[z][k] = 0.f;
+            if (F32) sum[z][k] = 0.f;
+        }
 
     // add `nb` <= 8 atoms from the queue's head to the brick
     auto add8 = [&](int head, int nb) {
@@ -169,6 +194,49 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         const float x[4] = {qa * weight(gq, pa, 0, fa.x, cx), qa * weight(gq + 8, pa, 0, fa.x, cx),
                             qb * weight(gq, pb, 0, fb.x, cx), qb * weight(gq + 8, pb, 0, fb.x, cx)};
         const float ya = weight(gq, pa, 8, fa.y, cy), yb = weight(gq, pb, 8, fb.y, cy);
+        if (F32) {
+            SpreadWeights& U = sh.xy[warp];
+            U.x[tq][gq] = x[0];
+            U.x[tq][gq + 8] = x[1];
+            U.x[tq + 4][gq] = x[2];
+            U.x[tq + 4][gq + 8] = x[3];
+            U.y[tq][gq] = ya;
+            U.y[tq + 4][gq] = yb;
+            __syncwarp();
+            #pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float4 wx = *reinterpret_cast<const float4*>(&U.x[k][4 * tq]);
+                const float wy = U.y[k][gq];
+                const float2 w0 = __fmul2_rn(make_float2(wx.x, wx.y), make_float2(wy, wy));
+                const float2 w1 = __fmul2_rn(make_float2(wx.z, wx.w), make_float2(wy, wy));
+                const float4 za = *reinterpret_cast<const float4*>(&W.z[k][0]);
+                const float4 zb = *reinterpret_cast<const float4*>(&W.z[k][4]);
+                const float wz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+                #pragma unroll
+                for (int z = 0; z < 8; ++z) {
+                    const float2 zz = make_float2(wz[z], wz[z]);
+                    const float2 r0 = __ffma2_rn(w0, zz, make_float2(acc[z][0], acc[z][1]));
+                    const float2 r1 = __ffma2_rn(w1, zz, make_float2(acc[z][2], acc[z][3]));
+                    acc[z][0] = r0.x;
+                    acc[z][1] = r0.y;
+                    acc[z][2] = r1.x;
+                    acc[z][3] = r1.y;
+                }
+            }
+            __syncwarp();
+            if ((++groups & 1) == 0)
+                #pragma unroll
+                for (int z = 0; z < 8; ++z)
+                    #pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        const float2 r = __fadd2_rn(make_float2(sum[z][k], sum[z][k + 1]),
+                                                    make_float2(acc[z][k], acc[z][k + 1]));
+                        sum[z][k] = r.x;
+                        sum[z][k + 1] = r.y;
+                        acc[z][k] = acc[z][k + 1] = 0.f;
+                    }
+            return;
+        }
         float xh[4], xl[4];
         #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -253,7 +321,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                     if (ok) {
                         const int q = (head + count + __popc(bal & ((1u << lane) - 1u))) & (kQueue - 1);
                         // (BF16 operands keep nothing of the fraction's last digits)
-                        W.f[q] = out == 2 ? make_float4(ux - fx, uy - fy, uz - fz, p.w)
+                        W.f[q] = !F32 && out == 2 ? make_float4(ux - fx, uy - fy, uz - fz, p.w)
                                           : make_float4(grid_frac(g.box, 0, p.x, fx), grid_frac(g.box, 1, p.y, fy),
                                                         grid_frac(g.box, 2, p.z, fz), p.w);
                         W.b[q] = (b0 + 32) | (b1 + 32) << 8 | (b2 + 32) << 16;
@@ -270,6 +338,11 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         }
         if (count > 0) add8(head, count);
     }
+    if (F32)
+        #pragma unroll
+        for (int z = 0; z < 8; ++z)
+            #pragma unroll
+            for (int k = 0; k < 4; ++k) acc[z][k] += sum[z][k];
 
     if (S > 1) {
         // add the bricks' shares in order of the split
@@ -295,12 +368,12 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         for (int z = 0; z < 8; ++z)
             #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int x = gq + 8 * (k >> 1), y = 2 * tq + (k & 1);
+                const int x = F32 ? 4 * tq + k : gq + 8 * (k >> 1), y = F32 ? gq : 2 * tq + (k & 1);
                 if (x >= ex || y >= ey || z >= ez) continue;
                 const size_t i = ((size_t)(oz + z) * n1 + (oy + y)) * n0 + (ox + x);
                 const float v = acc[z][k];
                 cs.add(v);
-                if (out == 0) {
+                if (F32) {
                     static_cast<float*>(rho)[i] = v;
                 } else if (out == 1) {
                     uint32_t hb;
@@ -313,7 +386,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                     static_cast<__nv_bfloat16*>(rho)[i] = hi;
                     static_cast<__nv_bfloat16*>(rho_lo)[i] = __float2bfloat16_rn(v - __bfloat162float(hi));
                 }
-                if (out != 0 && rho32) rho32[i] = v;
+                if (!F32 && rho32) rho32[i] = v;
             }
     }
     const double local = warp_sum(cs);
@@ -397,9 +470,10 @@ void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, vo
                    cudaStream_t st)
 {
     const int bx = bricks_along(g.box.n[0], kBrickX), by = bricks_along(g.box.n[1], kBrick);
-#define USR_SPREAD(S, W)                                                                                           \
-    launch_pdl(k_spread<S, W>, spread_ctas(g.box.n), 32 * W, 0, st, L.cpos, L.pstart, g, P, bx, by,                 \
+#define USR_SPREAD_FORM(S, W, F)                                                                                   \
+    launch_pdl(k_spread<S, W, F>, spread_ctas(g.box.n), 32 * W, 0, st, L.cpos, L.pstart, g, P, bx, by,              \
                bricks_of(g.box.n), split, rho, rho_lo, rho32, partial, counter, mean, status)
+#define USR_SPREAD(S, W) if (split == 0) USR_SPREAD_FORM(S, W, true); else USR_SPREAD_FORM(S, W, false)
     switch (splits_of(g.box.n)) {
         case 1: USR_SPREAD(1, kSpreadWarps); break;
         case 2: USR_SPREAD(2, kSpreadWarps); break;
@@ -407,6 +481,7 @@ void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, vo
         default: USR_SPREAD(8, 8); break;
     }
 #undef USR_SPREAD
+#undef USR_SPREAD_FORM
 }
 
 }  // namespace usr
