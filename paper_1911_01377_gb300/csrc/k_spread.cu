@@ -22,7 +22,7 @@
  *       4.6e-6, with blocks by 1.8e-6 (1.0e-6 is the method's own error).  Evaluations in the FP32 form with
  *       FMAs / on the tensor cores: 3,000 charges 70.3 / 71.0 us, 7,013 ions 90.9 / 92.7, slab 272 / 269.
  *       Up to 249 bricks eight warps share one and an SM gets at most two CTAs, so their registers are not capped
- *       at 128 (they would spill 108 bytes: 3,000 charges 71.8 us).
+ *       at 128 (3,000 charges 71.8 us with the cap).
  *
  * Every warp works by itself: it lists the atoms of the cells its brick's stencils can reach (rows of cells,
  * periodic images as separate rows), keeps those that do reach in a small queue in list order, and evaluates
@@ -139,6 +139,7 @@ template <int S, int WARPS, bool F32>
 __global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) k_spread(const float4* __restrict__ pos,
                                                         const int* __restrict__ pstart, GridArgs g, int P,
                                                         int bricks_x, int bricks_y, int bricks, int out,
+                                                        const ChargeSum* __restrict__ qsum,
                                                         void* __restrict__ rho, void* __restrict__ rho_lo,
                                                         float* __restrict__ rho32, double* __restrict__ partial,
                                                         unsigned int* __restrict__ counter,
@@ -338,6 +339,10 @@ __global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) 
         }
         if (count > 0) add8(head, count);
     }
+    // The operand splits keep a fixed number of digits of what they are given: rho's mean (the net charge over the
+    // grid, dropped as the k = 0 mode) is taken off before.  Any constant would do; the mean of what is written is
+    // measured below, and the x pass (or the first restriction) takes it off exactly.
+    const float m0 = F32 ? 0.f : __ll2float_rn((long long)qsum->sum) * exp2_int(-charge_bits(qsum->max)) * g.qmean;
     if (F32)
         #pragma unroll
         for (int z = 0; z < 8; ++z)
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) 
                 const int x = F32 ? 4 * tq + k : gq + 8 * (k >> 1), y = F32 ? gq : 2 * tq + (k & 1);
                 if (x >= ex || y >= ey || z >= ez) continue;
                 const size_t i = ((size_t)(oz + z) * n1 + (oy + y)) * n0 + (ox + x);
-                const float v = acc[z][k];
+                const float v = F32 ? acc[z][k] : acc[z][k] - m0;
                 cs.add(v);
                 if (F32) {
                     static_cast<float*>(rho)[i] = v;
@@ -465,14 +470,14 @@ int spread_ctas(const int* n)
     return (bricks_of(n) + nb - 1) / nb;
 }
 
-void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, void* rho,
+void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, const ChargeSum* qsum, void* rho,
                    void* rho_lo, float* rho32, double* partial, unsigned int* counter, double* mean, int* status,
                    cudaStream_t st)
 {
     const int bx = bricks_along(g.box.n[0], kBrickX), by = bricks_along(g.box.n[1], kBrick);
 #define USR_SPREAD_FORM(S, W, F)                                                                                   \
     launch_pdl(k_spread<S, W, F>, spread_ctas(g.box.n), 32 * W, 0, st, L.cpos, L.pstart, g, P, bx, by,              \
-               bricks_of(g.box.n), split, rho, rho_lo, rho32, partial, counter, mean, status)
+               bricks_of(g.box.n), split, qsum, rho, rho_lo, rho32, partial, counter, mean, status)
 #define USR_SPREAD(S, W) if (split == 0) USR_SPREAD_FORM(S, W, true); else USR_SPREAD_FORM(S, W, false)
     switch (splits_of(g.box.n)) {
         case 1: USR_SPREAD(1, kSpreadWarps); break;

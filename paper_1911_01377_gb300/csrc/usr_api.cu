@@ -69,6 +69,7 @@ struct usr_ctx {
     int *d_pstart = nullptr, *d_cperm = nullptr, *d_ccell = nullptr, *d_gfull = nullptr, *d_gpart = nullptr;
     int4* d_gdesc = nullptr;
     int* d_queue = nullptr;
+    usr::ChargeSum* d_qsum = nullptr;       // the charges' sum (tensor-core forms)
     float4 *d_cpos = nullptr, *d_bblo = nullptr, *d_bbhi = nullptr;
     // grids and convolution tables
     float *d_rho = nullptr, *d_X = nullptr, *d_Y = nullptr, *d_psi = nullptr;
@@ -143,7 +144,7 @@ void free_all(usr_ctx* c)
 {
     void* ptrs[] = {c->d_count, c->d_cell_of, c->d_slot, c->d_cell_start, c->d_unsorted, c->d_perm, c->d_status,
                     c->d_pstart, c->d_cperm, c->d_ccell, c->d_cpos, c->d_bblo, c->d_bbhi,
-                    c->d_wpos, c->d_spos, c->d_nacc, c->d_gfull, c->d_gpart, c->d_gdesc, c->d_queue, c->d_rho, c->d_X, c->d_Y, c->d_psi, c->d_Bx, c->d_Ay,
+                    c->d_wpos, c->d_spos, c->d_nacc, c->d_gfull, c->d_gpart, c->d_gdesc, c->d_queue, c->d_qsum, c->d_rho, c->d_X, c->d_Y, c->d_psi, c->d_Bx, c->d_Ay,
                     c->d_Az, c->d_wx, c->d_wy, c->d_wz, c->d_spread_partial, c->d_mean, c->d_gather_partial,
                     c->d_energy, c->d_netq, c->d_counters, c->d_in, c->d_out, c->d_near_dbg, c->d_far_dbg, c->d_far4,
                     c->d_psi_mean, c->d_ktab};
@@ -429,6 +430,8 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
     ENSURE(c->d_count, i4 * c->ncell);
     // the cell counters start at zero; every evaluation's scan leaves them zero again
     if (cudaMemsetAsync(c->d_count, 0, i4 * c->ncell, st) != cudaSuccess) return USR_ERR_CUDA;
+    ENSURE(c->d_qsum, sizeof(usr::ChargeSum));   // and so do the largest charge and their sum
+    if (cudaMemsetAsync(c->d_qsum, 0, sizeof(usr::ChargeSum), st) != cudaSuccess) return USR_ERR_CUDA;
     ENSURE(c->d_cell_start, i4 * (c->ncell + 1));
     ENSURE(c->d_pstart, i4 * (c->ncell + 1));
     ENSURE(c->d_cpos, f4 * ncl * 8);
@@ -701,6 +704,7 @@ void fill_args(usr_ctx* c)
     g.F0 = (float)P.F0;
     g.F0d = P.F0;
     g.wsum = (float)P.wsum;
+    g.qmean = (float)(P.wsum / ((double)P.n[0] * P.n[1] * P.n[2]));
 }
 
 usr_status check_device(const usr_ctx* c)
@@ -713,11 +717,12 @@ usr_status check_device(const usr_ctx* c)
 /* Cell list, 8-atom clusters, groups and zeroed accumulators. */
 void bin_and_cluster(usr_ctx* c, int n, const float4* xyzq, cudaStream_t st)
 {
+    usr::ChargeSum* qsum = c->tc ? c->d_qsum : nullptr;
     usr::launch_bin_list(n, xyzq, c->boxf, c->ncell, c->d_count, c->d_cell_of, c->d_slot, c->d_wpos, c->d_cell_start,
-                         c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, c->d_unsorted, c->d_status, st);
+                         c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, qsum, c->d_unsorted, c->d_status, st);
     usr::launch_clusters(n, c->boxf, c->ncell, c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_gdesc,
                          c->d_unsorted, c->d_wpos, c->d_slot, c->d_cpos, c->d_cperm, c->d_ccell, c->d_bblo, c->d_bbhi,
-                         c->d_nacc, c->max_clusters, c->max_groups, c->d_status, st);
+                         c->d_nacc, qsum, c->max_clusters, c->max_groups, c->d_status, st);
 }
 
 usr::ClusterList cluster_list(const usr_ctx* c)
@@ -834,11 +839,11 @@ usr_status run_eval(usr_ctx* c, int n, const float4* xyzq, float4* out, double* 
         NvtxRange r("usr: far chain (spread, convolutions, psi mean)");
         mark(3, sd);
         if (c->tc)
-            usr::launch_spread(P.P, cluster_list(c), c->grid, c->tc_bf16 ? 2 : 1, c->tcf.rho_hi,
+            usr::launch_spread(P.P, cluster_list(c), c->grid, c->tc_bf16 ? 2 : 1, c->d_qsum, c->tcf.rho_hi,
                                c->tcf.rho_lo, (c->vir || c->mlN > 0) ? c->d_rho32 : nullptr, c->d_spread_partial,
                                c->d_counters, c->d_mean, c->d_status, sd);
         else
-            usr::launch_spread(P.P, cluster_list(c), c->grid, 0, c->d_rho, nullptr, nullptr,
+            usr::launch_spread(P.P, cluster_list(c), c->grid, 0, c->d_qsum, c->d_rho, nullptr, nullptr,
                                c->d_spread_partial, c->d_counters, c->d_mean, c->d_status, sd);
         {
             NvtxRange rn("usr: near pairs");
@@ -1094,8 +1099,8 @@ extern "C" usr_status usr_debug_cells(usr_ctx* c, int n, const float* xyzq, int*
     if (n == 0) return USR_OK;
     cudaStream_t st = (cudaStream_t)stream;
     usr::launch_bin_list(n, (const float4*)xyzq, c->boxf, c->ncell, c->d_count, c->d_cell_of, c->d_slot, c->d_wpos,
-                         c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, c->d_unsorted, c->d_status,
-                         st);
+                         c->d_cell_start, c->d_pstart, c->d_gfull, c->d_gpart, c->d_queue, nullptr, c->d_unsorted,
+                         c->d_status, st);
     usr::launch_cell_sort(n, c->ncell, c->d_cell_start, c->d_unsorted, c->d_wpos, c->d_perm, c->d_spos, c->d_status, st);
     cudaMemcpyAsync(cell, c->d_cell_of, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(perm, c->d_perm, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st);

@@ -176,7 +176,26 @@ struct BoxF {
     int n[3];
 };
 
+/*
+ * The charges' sum in fixed point (integers: the same bits in any order), scaled by the largest of them: the cell
+ * counting takes the maximum into max_new, the scan moves it to max and zeroes max_new and sum, the clusters add
+ * their charges to sum in units of 2^-charge_bits(max).  2^28 charges of the largest size stay below 2^62.
+ */
+struct ChargeSum {
+    unsigned long long sum;
+    int max_new, max;         // float bits of a magnitude
+};
+
 #ifdef __CUDACC__
+/* Bits after the binary point, for a largest magnitude below 2^e: 34 - e (at most 100, so that the unit is a float). */
+__device__ __forceinline__ int charge_bits(int max)
+{
+    const int e = (max >> 23) - 126;
+    return min(34 - e, 100);
+}
+
+__device__ __forceinline__ float exp2_int(int k) { return __int_as_float((k + 127) << 23); }
+
 /*
  * Fractional grid coordinate of x on axis a, given cell = floor(x gs): x n / L - cell with one rounding of a number
  * below 1 (x gs alone carries 2^-24 of a coordinate up to n, which the stencil weights amplify).
@@ -242,6 +261,7 @@ struct GridArgs {
     float dfac[3];        // h / sigma_s^2: derivative factor
     float F0;             // self-interaction constant (per-atom potential)
     float wsum;           // sum of the spreading weights over a stencil
+    float qmean;          // rho's mean per unit of net charge
     const double* psi_mean;   // grid mean of psi (its k = 0 mode, zero up to rounding)
     double F0d;           // the same in FP64 (self energy)
 };
@@ -319,14 +339,14 @@ cudaError_t launch_bin(int n, const float4* xyzq, const BoxF& b, int ncell, int*
 /* The cell list (cell ids, counting sort, any order within a cell); each cell in the order of caller indices (the
    inspection entry points only); the 8-atom clusters. */
 void launch_bin_list(int n, const float4* xyzq, const BoxF& b, int ncell, int* count, int* cell_of, int* slot,
-                     float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue, int* unsorted,
-                     int* status, cudaStream_t st);
+                     float4* wpos, int* cell_start, int* pstart, int* gfull, int* gpart, int* queue,
+                     ChargeSum* qsum, int* unsorted, int* status, cudaStream_t st);
 void launch_cell_sort(int n, int ncell, const int* cell_start, const int* unsorted, const float4* wpos, int* perm,
                       float4* spos, int* status, cudaStream_t st);
 void launch_clusters(int n, const BoxF& b, int ncell, const int* cell_start, const int* pstart, const int* gfull,
                      const int* gpart, int4* gdesc, const int* unsorted, const float4* wpos, int* key, float4* cpos,
                      int* cperm, int* ccell, float4* bblo, float4* bbhi, unsigned long long* near_acc,
-                     int max_clusters, int max_groups, int* status, cudaStream_t st);
+                     ChargeSum* qsum, int max_clusters, int max_groups, int* status, cudaStream_t st);
 /* Upper bound of the half-list kernel's groups for n atoms in ncell cells; clusters per group. */
 int near_max_groups(int n, int ncell);
 int near_group_clusters();
@@ -339,9 +359,10 @@ void launch_near(int max_groups, int deg, const ClusterList& L, const NearArgs& 
 void set_near_ctas_per_sm(usr_ctx* c, int ctas_per_sm);
 void launch_pairs(int max_clusters, const ClusterList& L, const NearArgs& a, int* count,
                   unsigned long long* hash, int* status, cudaStream_t st);
-/* rho with its k = 0 mode still in it, as FP32 (split 0, rho) or a TF32 / BF16 operand split (1 / 2, rho and
-   rho_lo, and an FP32 copy in rho32 when that is non-null), and its grid mean through spread_ctas(n) partial sums */
-void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, void* rho,
+/* rho as FP32 (split 0, rho) or, less the mean that qsum gives, as a TF32 / BF16 operand split (1 / 2, rho and
+   rho_lo, and an FP32 copy in rho32 when that is non-null), and the grid mean of what was written through
+   spread_ctas(n) partial sums */
+void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, const ChargeSum* qsum, void* rho,
                    void* rho_lo, float* rho32, double* partial, unsigned int* counter, double* mean, int* status,
                    cudaStream_t st);
 int spread_ctas(const int* n);
