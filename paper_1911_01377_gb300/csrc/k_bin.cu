@@ -277,6 +277,18 @@ __device__ __forceinline__ int rank_of(const long long* k, int lo, int hi, long 
     return r;
 }
 
+/* The CTA's barrier; in the debug build, whether any thread found an index out of range. */
+__device__ __forceinline__ bool barrier_bad(bool bad)
+{
+#ifdef USR_DEBUG_BOUNDS
+    return __syncthreads_or(bad) != 0;
+#else
+    (void)bad;
+    __syncthreads();
+    return false;
+#endif
+}
+
 /*
  * The clusters of one cell per CTA, from the cell's entries in any order (k_place): the packing above, the padded
  * layout, each cluster's bounding box; also the descriptor of each of the cell's groups of gcl clusters, and the
@@ -340,6 +352,7 @@ __global__ void __launch_bounds__(256) k_cluster_build(const int* __restrict__ s
         for (int w = 1; w < threads >> 5; ++w) qs += qwarp[w];
         atomicAdd(&qsum->sum, (unsigned long long)qs);    // two's complement
     };
+    bool bad = false;                                     // (debug build) an entry of the cell is out of range
     if (m <= kTileMax) {
         const int ncl = pm >> 3;
         int sx = 1;                                       // slabs: the cube root of the clusters, rounded
@@ -348,6 +361,7 @@ __global__ void __launch_bounds__(256) k_cluster_build(const int* __restrict__ s
             long long key0 = LLONG_MAX;
             if (e < m) {
                 const int x = unsorted[s0 + e];
+                if (!USR_IN_BOUNDS(x, n, status)) { bad = true; continue; }
                 const float4 p = wpos[x];
                 key0 = tile_key(p.x - ox, x);
                 qs += __float2ll_rn(p.w * unit);
@@ -355,7 +369,7 @@ __global__ void __launch_bounds__(256) k_cluster_build(const int* __restrict__ s
             k0[e] = key0;
         }
         put_sum();
-        __syncthreads();
+        if (barrier_bad(bad)) return;
         add_sum();
         // each pass puts every atom at its place in the next order and stores its next key there
         for (int e = threadIdx.x; e < pm; e += threads) {
@@ -398,12 +412,13 @@ __global__ void __launch_bounds__(256) k_cluster_build(const int* __restrict__ s
         int* kk = key + s0;
         const int* xs = unsorted + s0;
         for (int e = threadIdx.x; e < m; e += threads) {
+            if (!USR_IN_BOUNDS(xs[e], n, status)) { bad = true; continue; }
             const float4 p = wpos[xs[e]];
             kk[e] = morton_key(p, ox, oy, oz, fx, fy, fz);
             qs += __float2ll_rn(p.w * unit);
         }
         put_sum();
-        __syncthreads();
+        if (barrier_bad(bad)) return;
         add_sum();
         // rank of (Morton code, caller index), four atoms to a thread, against a tile of the cell's keys at a time in
         // shared memory.  Bound: the m^2 comparisons.  Evaluations with 3,000 charges in one cell / 20,000 in eight:

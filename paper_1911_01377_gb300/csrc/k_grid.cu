@@ -269,7 +269,8 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
     for (int s0 = blockIdx.x * APC + warp * APW; s0 < ns; s0 += gridDim.x * APC) {
         const int s = s0 + slot;
         // lanes past APW x LPA hold no atom, and neither do the padding slots (near -1e6)
-        float4 p = slot < APW && s < ns ? cpos[s] : make_float4(-1.0e6f, 0.f, 0.f, 0.f);
+        float4 p = slot < APW && s < ns && USR_IN_BOUNDS(s, g.max_slots, status) ? cpos[s]
+                                                                                 : make_float4(-1.0e6f, 0.f, 0.f, 0.f);
         const bool have = p.x > -5.0e5f;
         if (!have) p = make_float4(0.f, 0.f, 0.f, 0.f);
         const float pc[3] = {p.x, p.y, p.z};
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
                 az += __shfl_down_sync(0xffffffffu, p3, o);
             }
         }
-        if (have && u == 0 && USR_IN_BOUNDS(s, g.max_slots, status)) {
+        if (have && u == 0) {
             const float qi = p.w;
             far4[s] = make_float4(-qi * ax, -qi * ay, -qi * az, aphi);
         }
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kGThreads, 8)
     for (int c0 = blockIdx.x * (kGWarps * per); c0 < ns; c0 += gridDim.x * (kGWarps * per)) {
         const int s1 = min(ns, c0 + kGWarps * per);
         for (int s = c0 + warp; s < s1; s += kGWarps) {
+            if (!USR_IN_BOUNDS(s, g.max_slots, status)) continue;
             const float4 p = cpos[s];
             if (p.x < -5.0e5f) continue;           // a padding slot (near -1e6)
             const float ux = p.x * g.box.gs[0], uy = p.y * g.box.gs[1], uz = p.z * g.box.gs[2];
@@ -501,7 +503,7 @@ __global__ void __launch_bounds__(kGThreads, 8)
             float v = (h3 ? k1 : k0) + t2;
             #pragma unroll
             for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if ((lane & 7) == 0 && USR_IN_BOUNDS(s, g.max_slots, status))
+            if ((lane & 7) == 0)
                 reinterpret_cast<float*>(far4 + s)[lane >> 3] = lane < 24 ? -p.w * v : v;
             __syncwarp();   // zw and zo are rewritten
         }
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(kThreads) k_combine(const float4* __restrict__
                                                       unsigned int* __restrict__ counter,
                                                       double* __restrict__ energy,
                                                       double* __restrict__ net_charge, int max_atoms,
-                                                      int* __restrict__ status)
+                                                      int max_slots, int* __restrict__ status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
     __shared__ double red[kWarps][4];
@@ -538,6 +540,7 @@ __global__ void __launch_bounds__(kThreads) k_combine(const float4* __restrict__
     CSum qn, qf, qq, qs;                              // sums of q phi_near, q phi_far, q^2, q
     const int ns = *nslots;
     for (int t = blockIdx.x * kThreads + threadIdx.x; t < ns; t += gridDim.x * kThreads) {
+        if (!USR_IN_BOUNDS(t, max_slots, status)) continue;
         const int i = cperm[t];
         const float4 nr = near_part(near_acc, t), f = far4[t];
         const float qi = cpos[t].w;
@@ -643,7 +646,7 @@ void launch_combine(int n, const ClusterList& L, int ncell, const unsigned long 
     const int nb = std::max(1, std::min(kCombineBlocks, (max_slots_of(n, ncell) + kThreads - 1) / kThreads));
     k_combine<<<nb, kThreads, 0, st>>>(L.cpos, L.cperm, L.pstart + ncell, near_acc, far4, g.F0, g.F0d, g.wsum,
                                        g.psi_mean, out, near_dbg, far_dbg, partial, counter, energy, net_charge, n,
-                                       status);
+                                       g.max_slots, status);
 }
 
 }  // namespace usr

@@ -206,10 +206,12 @@ struct NearShared {
     int off[kSplitCells], end[kSplitCells];
 };
 
-/* The group of work unit u into d (a warp's next unit, or none when u >= units). */
-__device__ __forceinline__ int near_next(const ClusterList& L, const NearArgs& a, int u, int units, int4& d)
+/* The group of work unit u into d (a warp's next unit); units when there is none. */
+__device__ __forceinline__ int near_next(const ClusterList& L, const NearArgs& a, int u, int units, int4& d,
+                                         int* __restrict__ status)
 {
-    if (u < units) d = L.gdesc[u / kNearSplits];
+    if (u >= units || !USR_IN_BOUNDS(u / kNearSplits, a.max_groups, status)) return units;
+    d = L.gdesc[u / kNearSplits];
     return u;
 }
 
@@ -285,7 +287,7 @@ __device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& 
     V.xx = V.yy = V.zz = V.xy = V.xz = V.yz = dup(0.f);
     const bool tri_a = jl > gi, tri_b = jl > gi + 4;
     const bool b1 = (lane & 16) != 0, b0 = (lane & 8) != 0;
-    if (total == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn);
+    if (total == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn, status);
     // clusters of the unit's own cell come first: candidate t < GI is cluster c0 + t, one of the group's own
     const int nown = nb0 == 13 ? ni : 0;
     int ends[kSplitCells];                 // uniform copies
@@ -322,7 +324,7 @@ __device__ __forceinline__ void near_unit(const ClusterList& L, const NearArgs& 
                 }
             }
         }
-        if (tb == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn);
+        if (tb == 0) next = near_next(L, a, __shfl_sync(0xffffffffu, ticket, 0), units, dn, status);
         unsigned int bal = __ballot_sync(0xffffffffu, m != 0);
         if (!bal) continue;
         // the surviving j-clusters; the next one's atoms are loaded while this one's steps run
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(128, USR_NEAR_MINB) k_near_half(ClusterList L,
     int u = 0;
     if (lane == 0) u = atomicAdd(queue, 1);
     int4 d = make_int4(0, 0, 0, 0);
-    u = near_next(L, a, __shfl_sync(0xffffffffu, u, 0), units, d);
+    u = near_next(L, a, __shfl_sync(0xffffffffu, u, 0), units, d, status);
     while (u < units) {
         const int sub = u % kNearSplits, nb0 = 13 + sub * kSplitCells, nb1 = min(27, nb0 + kSplitCells);
         if (!USR_IN_BOUNDS(d.x + d.z - 1, a.max_clusters, status)) return;

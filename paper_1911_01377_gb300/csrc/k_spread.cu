@@ -307,13 +307,16 @@ __global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) 
                 // this warp's chunks of 32 atoms: every S-th of the list
                 int base = 32 * ((split - turn) & (S - 1));
                 turn += (rc + 31) >> 5;
-                float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (base + lane < rc) next = pos[rf + base + lane];
+                // atom k of the run; past its end a padding slot (these lie near -1e6)
+                auto fetch = [&](int k) {
+                    return k < rc && USR_IN_BOUNDS(rf + k, g.max_slots, status) ? pos[rf + k]
+                                                                                : make_float4(-1.0e6f, 0.f, 0.f, 0.f);
+                };
+                float4 next = fetch(base + lane);
                 for (; base < rc; base += 32 * S) {
                     const float4 p = next;
-                    // a padding slot lies near -1e6
-                    bool ok = base + lane < rc && p.x > -5.0e5f && USR_IN_BOUNDS(rf + base + lane, g.max_slots, status);
-                    if (base + 32 * S + lane < rc) next = pos[rf + base + 32 * S + lane];
+                    bool ok = p.x > -5.0e5f;
+                    next = fetch(base + 32 * S + lane);
                     const float ux = p.x * g.box.gs[0], uy = p.y * g.box.gs[1], uz = p.z * g.box.gs[2];
                     const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
                     const int b0 = (int)fx + rx, b1 = (int)fy + ry, b2 = (int)fz + rz;

@@ -1148,6 +1148,18 @@ extern "C" usr_status usr_debug_inject_timeout(usr_ctx* c, int on)
     return USR_OK;
 }
 
+#ifdef USR_DEBUG_BOUNDS
+/* Debug build only, for its tests: the checks take max_slots cluster slots and max_groups groups as the buffers'
+   sizes (each only lowered; the buffers stay as they are). */
+extern "C" usr_status usr_debug_limit_bounds(usr_ctx* c, int max_slots, int max_groups)
+{
+    if (!c || max_slots < 0 || max_groups < 0) return USR_ERR_ARG;
+    c->grid.max_slots = std::min(c->grid.max_slots, max_slots);
+    c->near.max_groups = std::min(c->near.max_groups, max_groups);
+    return USR_OK;
+}
+#endif
+
 extern "C" usr_status usr_set_keep_parts(usr_ctx* c, int on)
 {
     if (!c) return USR_ERR_ARG;
