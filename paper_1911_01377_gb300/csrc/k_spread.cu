@@ -268,17 +268,12 @@ __global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) 
     };
 
     if (owns) {
-        // cells (unwrapped) that hold atoms whose stencil reaches [o, o + e): grid coordinates o - H .. o + e + H - 1
-        // (the margin covers the single-precision rounding of cell ids and grid coordinates, below 2e-4 cells)
-        int c0[3], c1[3];
+        int c0[3], c1[3];                                 // cells that may hold atoms whose stencil reaches the brick
         {
             const int o[3] = {ox, oy, oz}, e[3] = {ex, ey, ez};
             #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const float r = (float)g.box.nc[a] / (float)g.box.n[a];
-                c0[a] = (int)floorf((float)(o[a] - H) * r - 1.0e-3f);
-                c1[a] = (int)floorf((float)(o[a] + e[a] + H - 1) * r + 1.0e-3f);
-            }
+            for (int a = 0; a < 3; ++a)
+                spread_cells(o[a], e[a], H, g.box.n[a], g.box.nc[a], kSpreadMargin, &c0[a], &c1[a]);
         }
         const int ny = c1[1] - c0[1] + 1, nz = c1[2] - c0[2] + 1;
         const int px = floor_div(c0[0], ncx), npx = floor_div(c1[0], ncx) - px + 1;   // periods the x range touches

@@ -5,6 +5,7 @@
  */
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <new>
 #include <vector>
@@ -175,6 +176,27 @@ struct BoxF {
     int nc[3];
     int n[3];
 };
+
+#ifdef __CUDACC__
+#define USR_HD __host__ __device__ __forceinline__
+#else
+#define USR_HD inline
+#endif
+
+/*
+ * Cells (unwrapped) along an axis of n grid points and nc cells that may hold atoms whose stencil of 2 H points reaches
+ * the points [o, o + e): grid coordinates o - H to o + e + H - 1, that is cells floor((o - H) nc / n) to
+ * floor((o + e + H - 1) nc / n).  The margin (in cells) covers the single-precision rounding here, of cell ids and of
+ * grid coordinates; the bounds of these add to 7e-4 cells at 4,096 points per axis.  A CPU test checks the range
+ * against every single-precision coordinate (margins up to 1e-4 fail it, 2e-4 passes).
+ */
+constexpr float kSpreadMargin = 1.0e-3f;
+USR_HD void spread_cells(int o, int e, int H, int n, int nc, float margin, int* c0, int* c1)
+{
+    const float r = (float)nc / (float)n;
+    *c0 = (int)floorf(fmaf((float)(o - H), r, -margin));
+    *c1 = (int)floorf(fmaf((float)(o + e + H - 1), r, margin));
+}
 
 /*
  * The charges' sum in fixed point (integers: the same bits in any order), scaled by the largest of them: the cell
