@@ -20,9 +20,9 @@
  *       tensor-core form does not cancel over the net charge of a region: with it, the far potential of a drop
  *       of water in vacuum (6,000 charges in 90 A) was off by 6.2e-6 of its norm, with FMAs in one chain by
  *       4.6e-6, with blocks by 1.8e-6 (1.0e-6 is the method's own error).  Evaluations in the FP32 form with
- *       FMAs / on the tensor cores: 3,000 charges 70.3 / 71.0 us, 7,013 ions 90.9 / 92.7, slab 272 / 269.
- *       Up to 249 bricks eight warps share one and an SM gets at most two CTAs, so their registers are not capped
- *       at 128 (3,000 charges 71.8 us with the cap).
+ *       FMAs / on the tensor cores: 3,000 charges 72.1 / 72.1 us, 7,013 ions 93.0 / 92.9, slab 273 / 269, 200 k
+ *       charges 932 / 908.  (With more than 128 registers where eight warps share a brick, small systems take 1 to 2
+ *       us less, and 6,400 charges at r_c = 13 A 114 us instead of 103: the pair kernel's CTAs must wait.)
  *
  * Every warp works by itself: it lists the atoms of the cells its brick's stencils can reach (rows of cells,
  * periodic images as separate rows), keeps those that do reach in a small queue in list order, and evaluates
@@ -136,7 +136,7 @@ struct SpreadShared {
 /* out: 0 FP32 rho; 1 and 2 the operand split of the tensor-core convolutions, rho = hi + lo with hi rounded to
    TF32 (1) or BF16 (2).  rho32: FP32 copy beside a split (may be null). */
 template <int S, int WARPS, bool F32>
-__global__ void __launch_bounds__(32 * WARPS, (F32 && S == 8 ? 8 : 16) / WARPS) k_spread(const float4* __restrict__ pos,
+__global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4* __restrict__ pos,
                                                         const int* __restrict__ pstart, GridArgs g, int P,
                                                         int bricks_x, int bricks_y, int bricks, int out,
                                                         const ChargeSum* __restrict__ qsum,
