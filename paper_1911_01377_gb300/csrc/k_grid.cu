@@ -66,13 +66,6 @@ __device__ __forceinline__ double warp_sum_c(CSum cs)
     return cs.value();
 }
 
-__device__ __forceinline__ float warp_sum_f(float v)
-{
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 /* Periodic wrap of a grid index that lies within two periods of [0, n). */
 __device__ __forceinline__ int wrap_once(int v, int n)
 {
@@ -84,26 +77,20 @@ __device__ __forceinline__ int wrap_once(int v, int n)
 }  // namespace
 
 /*
- * Grid mean of psi.  Exact arithmetic gives psi no k = 0 mode (rho has its
- * mean removed and the kernels are convolutions), but the FP32 rounding of
- * rho's mean removal leaves a tiny mean that the wide Gaussian terms amplify
- * by their k = 0 transform; the gather subtracts the mean measured here.
- * Fixed-order FP64 partial sums, the last CTA finishes.
+ * out = scale * sum_g a_g b_g (the virial's products of rho with the strain derivatives of psi): compensated FP32
+ * within a thread, FP64 partial sums per CTA in a fixed order, the last CTA finishes.
  */
-__global__ void __launch_bounds__(256) k_grid_mean(long long G, const float* __restrict__ psi,
-                                                   const float* __restrict__ w, double scale,
-                                                   double* __restrict__ partial, unsigned int* __restrict__ counter,
-                                                   double* __restrict__ mean)
+__global__ void __launch_bounds__(256) k_grid_dot(long long G, const float* __restrict__ a,
+                                                  const float* __restrict__ b, double scale,
+                                                  double* __restrict__ partial, unsigned int* __restrict__ counter,
+                                                  double* __restrict__ out)
 {
     __shared__ double red[8];
     __shared__ int is_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     CSum cs;
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < G; i += (long long)gridDim.x * 256)
-        if (w)
-            cs.add_product(psi[i], w[i]);
-        else
-            cs.add(psi[i]);
+        cs.add_product(a[i], b[i]);
     double s = warp_sum_c(cs);
     if (lane == 0) red[warp] = s;
     __syncthreads();
@@ -125,18 +112,17 @@ __global__ void __launch_bounds__(256) k_grid_mean(long long G, const float* __r
         if (threadIdx.x == 0) {
             double u = 0.0;
             for (int w = 0; w < 8; ++w) u += red[w];
-            *mean = u * scale;
+            *out = u * scale;
             *counter = 0u;
         }
     }
 }
 
-/* out = scale * sum_g a_g b_g in FP64, fixed order (the virial's grid dot products). */
 void launch_grid_dot(const GridArgs& g, const float* a, const float* b, double scale, double* partial,
                      unsigned int* counter, double* out, cudaStream_t st)
 {
     const long long G = (long long)g.box.n[0] * g.box.n[1] * g.box.n[2];
-    k_grid_mean<<<kGridMeanBlocks, 256, 0, st>>>(G, a, b, scale, partial, counter, out);
+    k_grid_dot<<<kGridDotBlocks, 256, 0, st>>>(G, a, b, scale, partial, counter, out);
 }
 
 /*
@@ -373,32 +359,22 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
  * equal (130 against 124 us for 200 k charges) and with 8, four points to a lane, this form is slower (44 against
  * 35 us on the slab): the weights then cost more than the rows.
  */
-template <int P, int V>
+template <int P>
 struct GatherShape {
-    static constexpr int NP = (P + 2 * (V - 1)) / V;              // lanes per row: P points at any offset mod V
+    static constexpr int NP = (P + 2) / 2;                        // lanes per row: P points at any offset mod 2
     static constexpr int R = 32 / NP < P ? 32 / NP : P;           // rows side by side
     static constexpr int BL = (P + R - 1) / R;                    // rows per lane
 };
 
-template <int V>
-struct VecOf;
-template <>
-struct VecOf<1> { typedef float T; };
-template <>
-struct VecOf<2> { typedef float2 T; };
-template <>
-struct VecOf<4> { typedef float4 T; };
-
-template <int P, int V>
+template <int P>
 __global__ void __launch_bounds__(kGThreads, 8)
-    k_gather_wide(const float4* __restrict__ cpos, const int* __restrict__ nslots, int per, const float* __restrict__ psi, GridArgs g,
-             float4* __restrict__ far4, double* __restrict__ partial, unsigned int* __restrict__ counter,
-             double* __restrict__ psi_mean, int* __restrict__ status)
+    k_gather_wide(const float4* __restrict__ cpos, const int* __restrict__ nslots, int per,
+                  const float* __restrict__ psi, GridArgs g, float4* __restrict__ far4, double* __restrict__ partial,
+                  unsigned int* __restrict__ counter, double* __restrict__ psi_mean, int* __restrict__ status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
     constexpr int H = P / 2;
-    typedef GatherShape<P, V> Sh;
-    typedef typename VecOf<V>::T Vec;
+    typedef GatherShape<P> Sh;
     __shared__ float2 zw[kGWarps][P];          // z weight and its derivative factor
     __shared__ unsigned int zo[kGWarps][P];    // offset of the plane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -428,10 +404,10 @@ __global__ void __launch_bounds__(kGThreads, 8)
                 zo[warp][lane] = (unsigned int)wrap_once(b2 + lane, n2) * plane;
             }
             // this lane's x points (weight 0 outside the stencil and for lanes past the last row)
-            const int xs = (b0 & ~(V - 1)) + V * slot;
-            float wx[V], dx[V];
+            const int xs = (b0 & ~1) + 2 * slot;
+            float wx[2], dx[2];
             #pragma unroll
-            for (int v = 0; v < V; ++v) {
+            for (int v = 0; v < 2; ++v) {
                 const int k = xs + v - b0;
                 const float d = (float)(k - H + 1) - tx;
                 wx[v] = k >= 0 && k < P && row < Sh::R ? __expf(-d * d * g.hh[0]) : 0.f;
@@ -449,46 +425,26 @@ __global__ void __launch_bounds__(kGThreads, 8)
                 off[b] = (unsigned int)wrap_once(b1 + (j < P ? j : 0), n1) * (unsigned int)n0 + xo;
             }
             __syncwarp();
-            float c0v[Sh::BL][V], c1v[Sh::BL][V];
+            float2 c0v[Sh::BL], c1v[Sh::BL];
             #pragma unroll
-            for (int b = 0; b < Sh::BL; ++b)
-                #pragma unroll
-                for (int v = 0; v < V; ++v) c0v[b][v] = c1v[b][v] = 0.f;
+            for (int b = 0; b < Sh::BL; ++b) c0v[b] = c1v[b] = make_float2(0.f, 0.f);
             #pragma unroll
             for (int k = 0; k < P; ++k) {
                 const float2 w = zw[warp][k];
                 const unsigned int z = zo[warp][k];
                 #pragma unroll
                 for (int b = 0; b < Sh::BL; ++b) {
-                    const Vec q = __ldg(reinterpret_cast<const Vec*>(psi + (z + off[b])));
-                    const float* f = reinterpret_cast<const float*>(&q);
-                    if (V == 1) {
-                        c0v[b][0] = fmaf(w.x, f[0], c0v[b][0]);
-                        c1v[b][0] = fmaf(w.y, f[0], c1v[b][0]);
-                    } else {
-                        #pragma unroll
-                        for (int v = 0; v + 1 < V; v += 2) {
-                            const float2 f2 = make_float2(f[v], f[v + 1]);
-                            const float2 r0 = __ffma2_rn(make_float2(w.x, w.x), f2, make_float2(c0v[b][v], c0v[b][v + 1]));
-                            const float2 r1 = __ffma2_rn(make_float2(w.y, w.y), f2, make_float2(c1v[b][v], c1v[b][v + 1]));
-                            c0v[b][v] = r0.x;
-                            c0v[b][v + 1] = r0.y;
-                            c1v[b][v] = r1.x;
-                            c1v[b][v + 1] = r1.y;
-                        }
-                    }
+                    const float2 f = __ldg(reinterpret_cast<const float2*>(psi + (z + off[b])));
+                    c0v[b] = __ffma2_rn(make_float2(w.x, w.x), f, c0v[b]);
+                    c1v[b] = __ffma2_rn(make_float2(w.y, w.y), f, c1v[b]);
                 }
             }
             float aphi = 0.f, ax = 0.f, ay = 0.f, az = 0.f;
             #pragma unroll
             for (int b = 0; b < Sh::BL; ++b) {
-                float r0 = 0.f, r1 = 0.f, r2 = 0.f;
-                #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    r0 = fmaf(wx[v], c0v[b][v], r0);
-                    r1 = fmaf(dx[v], c0v[b][v], r1);
-                    r2 = fmaf(wx[v], c1v[b][v], r2);
-                }
+                const float r0 = fmaf(wx[1], c0v[b].y, wx[0] * c0v[b].x);
+                const float r1 = fmaf(dx[1], c0v[b].y, dx[0] * c0v[b].x);
+                const float r2 = fmaf(wx[1], c1v[b].y, wx[0] * c1v[b].x);
                 aphi = fmaf(wy[b], r0, aphi);
                 ax = fmaf(wy[b], r1, ax);
                 ay = fmaf(dy[b], r0, ay);
@@ -615,7 +571,7 @@ static void gather_wide(int n, const ClusterList& L, int ncell, const float* psi
     // slots per warp and pass: up to 8 neighbours (their rows overlap in L1), fewer when that would leave warps idle
     const int slots = max_slots_of(n, ncell), per = std::max(1, std::min(8, slots / (kGWarps * kGatherBlocks)));
     const int nb = std::max(1, std::min(kGatherBlocks, (slots + kGWarps * per - 1) / (kGWarps * per)));
-    launch_with(-1, k_gather_wide<P, 2>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, per, psi, g, far4, partial,
+    launch_with(-1, k_gather_wide<P>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, per, psi, g, far4, partial,
                 counter, psi_mean, status);
 }
 

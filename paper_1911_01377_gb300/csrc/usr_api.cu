@@ -282,7 +282,7 @@ double usr::plan_device_bytes(const Plan& P)
     b += 4 * G + 8 * (nsb + kGatherBlocks + 4 * kCombineBlocks) + 8 * 11;
     if (P.p.virial) {   // six FP32 table sets, their inputs, two FP32 grids, warp slots, FP32 scratch grids
         b += 6 * 4 * N * (nx * nx + ny * ny + nz * nz + nx + ny + nz) + 6 * 8 * (3 * N * nmax + 4 * N);
-        b += 8 * G + 48 * near_units((int)ngr) + 8 * (16 + kGridMeanBlocks);
+        b += 8 * G + 48 * near_units((int)ngr) + 8 * (16 + kGridDotBlocks);
         if (tc) b += 4 * G * (1 + 2 * N);
     }
     if (P.Nc > 0) {   // multilevel: weights, coarse tables and their input, scratch, FP32 rho copy (tensor cores)
@@ -502,7 +502,7 @@ usr_status configure_plan(usr_ctx* c, const Plan& np, cudaStream_t st)
         ENSURE(c->d_rho32, fl * G);
         ENSURE(c->d_vnear, db * 6 * usr::near_units(c->max_groups));
         ENSURE(c->d_vdot, db * 6);
-        ENSURE(c->d_vpart, db * usr::kGridMeanBlocks);
+        ENSURE(c->d_vpart, db * usr::kGridDotBlocks);
         ENSURE(c->d_W, db * 9);
         for (int cmp = 0; cmp < 6; ++cmp) {
             ENSURE(c->d_vtab[cmp][0], fl * nx * N * nx);

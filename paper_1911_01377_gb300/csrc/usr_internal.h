@@ -28,7 +28,7 @@ constexpr long long kMaxGridPoints = (1LL << 31) - 1;   // grid points at most (
 constexpr int kMaxAtoms = 1 << 28;  // atoms per context at most (32-bit cluster-slot indices keep headroom)
 constexpr double kMaxBox = 1.0e5;   // box side at most (Angstrom): the pair kernel's padding rows, at -1e6 A and
                                     // beyond, then stay more than 7e5 A from every atom and periodic image
-constexpr int kGridMeanBlocks = 304;   // CTAs of the grid-mean reduction (two per SM)
+constexpr int kGridDotBlocks = 304;    // CTAs of the virial's grid products (two per SM)
 constexpr int kCombineBlocks = 608;    // CTAs of the near + far combination at most (four per SM)
 
 /*
