@@ -10,19 +10,21 @@
  * and their y weights times the z weight of plane z (8 atoms x 8 points) for each of its 8 planes, with the
  * brick's sums in registers.  Two forms:
  *
- *   split forms (TF32x3 and BF16x3 convolutions)  on the tensor cores (mma.sync m16n8k8).  The operands are
- *       split into TF32 high and low parts (to nearest) and three products are accumulated in FP32, which keeps
- *       about 22 bits of each factor; the MMA truncates its sums, so a brick's sums carry a bias of about 1e-7.
- *       The tcgen05 form would need the y-z products in shared memory, 256 bytes per atom and plane; here they
- *       are formed in registers.
- *   F32 (FP32 convolutions)  two-wide FP32 FMAs, a lane four x points of one y in every plane, in blocks of 16
- *       atoms that are summed apart (a point of a 12-point stencil receives about 170 terms).  The bias of the
- *       tensor-core form does not cancel over the net charge of a region: with it, the far potential of a drop
- *       of water in vacuum (6,000 charges in 90 A) was off by 6.2e-6 of its norm, with FMAs in one chain by
- *       4.6e-6, with blocks by 1.8e-6 (1.0e-6 is the method's own error).  Evaluations in the FP32 form with
- *       FMAs / on the tensor cores: 3,000 charges 72.1 / 72.1 us, 7,013 ions 93.0 / 92.9, slab 273 / 269, 200 k
- *       charges 932 / 908.  (With more than 128 registers where eight warps share a brick, small systems take 1 to 2
- *       us less, and 6,400 charges at r_c = 13 A 114 us instead of 103: the pair kernel's CTAs must wait.)
+ *   tensor cores (mma.sync m16n8k8): the split forms (TF32x3 and BF16x3 convolutions) with 8 and 10 points.  The
+ *       operands are split into TF32 high and low parts (to nearest) and three products are accumulated in FP32,
+ *       which keeps about 22 bits of each factor; the MMA truncates its sums, so a brick's sums carry a bias of
+ *       about 1e-7.  The tcgen05 form would need the y-z products in shared memory, 256 bytes per atom and plane;
+ *       here they are formed in registers.
+ *   FMA: the FP32 form, and every form from 12 points on.  Two-wide FP32 FMAs, a lane four x points of one y in
+ *       every plane, in blocks of 16 atoms that are summed apart (a point of a 12-point stencil receives about 170
+ *       terms).  The tensor cores' bias does not cancel over the net charge of a region: with them, the far
+ *       potential of a drop of water in vacuum (6,000 charges in 90 A) was off by 6.2e-6 of its norm, with FMAs
+ *       in one chain by 4.6e-6, with blocks by 1.8e-6, 1.0e-6 of which is the method's own error at 12 points (in
+ *       TF32x3 5.0e-6 and 1.8e-6; with 10 points the stencil itself leaves 4e-5).  Evaluations with FMAs / on the
+ *       tensor cores: FP32 form, 3,000 charges 72.1 / 72.1 us, 7,013 ions 93.0 / 92.9, slab 273 / 269, 200 k
+ *       charges 932 / 908; TF32x3, 60,000 ions at 16 points 344 / 327.  (With more than 128 registers where eight
+ *       warps share a brick, small systems take 1 to 2 us less, and 6,400 charges at r_c = 13 A 114 us instead of
+ *       103: the pair kernel's CTAs must wait.)
  *
  * Every warp works by itself: it lists the atoms of the cells its brick's stencils can reach (rows of cells,
  * periodic images as separate rows), keeps those that do reach in a small queue in list order, and evaluates
@@ -115,17 +117,17 @@ struct SpreadWarp {
     float z[8][kBrick];      // z weights of the current eight atoms
 };
 
-/* The FP32 form's further weights of the current eight atoms (rows of x weights 24 floats apart: a warp's stores of
+/* The FMA form's further weights of the current eight atoms (rows of x weights 24 floats apart: a warp's stores of
    four rows then touch each bank once). */
 struct SpreadWeights {
     float x[8][kBrickX + 8];
     float y[8][kBrick];
 };
 
-template <int S, int WARPS, bool F32>
+template <int S, int WARPS, bool FMA>
 struct SpreadShared {
     SpreadWarp w[WARPS];
-    SpreadWeights xy[F32 ? WARPS : 1];
+    SpreadWeights xy[FMA ? WARPS : 1];
     float4 share[S > 1 ? (WARPS - WARPS / S) * 256 : 1];   // bricks' shares of the splits after the first
     double red[WARPS];
     int is_last;
@@ -135,7 +137,7 @@ struct SpreadShared {
 
 /* out: 0 FP32 rho; 1 and 2 the operand split of the tensor-core convolutions, rho = hi + lo with hi rounded to
    TF32 (1) or BF16 (2).  rho32: FP32 copy beside a split (may be null). */
-template <int S, int WARPS, bool F32>
+template <int S, int WARPS, bool FMA>
 __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4* __restrict__ pos,
                                                         const int* __restrict__ pstart, GridArgs g, int P,
                                                         int bricks_x, int bricks_y, int bricks, int out,
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
     constexpr int NB = WARPS / S;
-    __shared__ __align__(16) SpreadShared<S, WARPS, F32> sh;
+    __shared__ __align__(16) SpreadShared<S, WARPS, FMA> sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = P / 2;
     const int n0 = g.box.n[0], n1 = g.box.n[1], n2 = g.box.n[2];
@@ -163,16 +165,16 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
     // exp(-d^2 hh) = 2^(d^2 c)
     const float kl = -1.4426950408889634f;
     const float cx = g.hh[0] * kl, cy = g.hh[1] * kl, cz = g.hh[2] * kl;
-    // per plane z, the points (x, y): (gq, 2 tq), (gq, 2 tq + 1), (gq + 8, 2 tq), (gq + 8, 2 tq + 1); F32: (4 tq, gq)
+    // per plane z, the points (x, y): (gq, 2 tq), (gq, 2 tq + 1), (gq + 8, 2 tq), (gq + 8, 2 tq + 1); FMA: (4 tq, gq)
     // .. (4 tq + 3, gq), acc holds the atoms since the last fold into sum
-    float acc[8][4], sum[F32 ? 8 : 1][4];
+    float acc[8][4], sum[FMA ? 8 : 1][4];
     int groups = 0;
     #pragma unroll
     for (int z = 0; z < 8; ++z)
         #pragma unroll
         for (int k = 0; k < 4; ++k) {
             acc[z][k] = 0.f;
-            if (F32) sum[z][k] = 0.f;
+            if (FMA) sum[z][k] = 0.f;
         }
 
     // add `nb` <= 8 atoms from the queue's head to the brick
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         const float x[4] = {qa * weight(gq, pa, 0, fa.x, cx), qa * weight(gq + 8, pa, 0, fa.x, cx),
                             qb * weight(gq, pb, 0, fb.x, cx), qb * weight(gq + 8, pb, 0, fb.x, cx)};
         const float ya = weight(gq, pa, 8, fa.y, cy), yb = weight(gq, pb, 8, fb.y, cy);
-        if (F32) {
+        if (FMA) {
             SpreadWeights& U = sh.xy[warp];
             U.x[tq][gq] = x[0];
             U.x[tq][gq + 8] = x[1];
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                     if (ok) {
                         const int q = (head + count + __popc(bal & ((1u << lane) - 1u))) & (kQueue - 1);
                         // (BF16 operands keep nothing of the fraction's last digits)
-                        W.f[q] = !F32 && out == 2 ? make_float4(ux - fx, uy - fy, uz - fz, p.w)
+                        W.f[q] = out == 2 ? make_float4(ux - fx, uy - fy, uz - fz, p.w)
                                           : make_float4(grid_frac(g.box, 0, p.x, fx), grid_frac(g.box, 1, p.y, fy),
                                                         grid_frac(g.box, 2, p.z, fz), p.w);
                         W.b[q] = (b0 + 32) | (b1 + 32) << 8 | (b2 + 32) << 16;
@@ -340,8 +342,8 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
     // The operand splits keep a fixed number of digits of what they are given: rho's mean (the net charge over the
     // grid, dropped as the k = 0 mode) is taken off before.  Any constant would do; the mean of what is written is
     // measured below, and the x pass (or the first restriction) takes it off exactly.
-    const float m0 = F32 ? 0.f : __ll2float_rn((long long)qsum->sum) * exp2_int(-charge_bits(qsum->max)) * g.qmean;
-    if (F32)
+    const float m0 = out == 0 ? 0.f : __ll2float_rn((long long)qsum->sum) * exp2_int(-charge_bits(qsum->max)) * g.qmean;
+    if (FMA)
         #pragma unroll
         for (int z = 0; z < 8; ++z)
             #pragma unroll
@@ -371,12 +373,12 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
         for (int z = 0; z < 8; ++z)
             #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int x = F32 ? 4 * tq + k : gq + 8 * (k >> 1), y = F32 ? gq : 2 * tq + (k & 1);
+                const int x = FMA ? 4 * tq + k : gq + 8 * (k >> 1), y = FMA ? gq : 2 * tq + (k & 1);
                 if (x >= ex || y >= ey || z >= ez) continue;
                 const size_t i = ((size_t)(oz + z) * n1 + (oy + y)) * n0 + (ox + x);
-                const float v = F32 ? acc[z][k] : acc[z][k] - m0;
+                const float v = acc[z][k] - m0;
                 cs.add(v);
-                if (F32) {
+                if (out == 0) {
                     static_cast<float*>(rho)[i] = v;
                 } else if (out == 1) {
                     uint32_t hb;
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_spread(const float4*
                     static_cast<__nv_bfloat16*>(rho)[i] = hi;
                     static_cast<__nv_bfloat16*>(rho_lo)[i] = __float2bfloat16_rn(v - __bfloat162float(hi));
                 }
-                if (!F32 && rho32) rho32[i] = v;
+                if (out != 0 && rho32) rho32[i] = v;
             }
     }
     const double local = warp_sum(cs);
@@ -473,10 +475,11 @@ void launch_spread(int P, const ClusterList& L, const GridArgs& g, int split, co
                    cudaStream_t st)
 {
     const int bx = bricks_along(g.box.n[0], kBrickX), by = bricks_along(g.box.n[1], kBrick);
+    const bool fma = split == 0 || P >= 12;   // 12 points and more resolve what the tensor cores' sums lack (above)
 #define USR_SPREAD_FORM(S, W, F)                                                                                   \
     launch_pdl(k_spread<S, W, F>, spread_ctas(g.box.n), 32 * W, 0, st, L.cpos, L.pstart, g, P, bx, by,              \
                bricks_of(g.box.n), split, qsum, rho, rho_lo, rho32, partial, counter, mean, status)
-#define USR_SPREAD(S, W) if (split == 0) USR_SPREAD_FORM(S, W, true); else USR_SPREAD_FORM(S, W, false)
+#define USR_SPREAD(S, W) if (fma) USR_SPREAD_FORM(S, W, true); else USR_SPREAD_FORM(S, W, false)
     switch (splits_of(g.box.n)) {
         case 1: USR_SPREAD(1, kSpreadWarps); break;
         case 2: USR_SPREAD(2, kSpreadWarps); break;
