@@ -537,7 +537,7 @@ def run_gpu(args):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": "f32 pairs/spreading, bf16x3 tensor-core convolutions with f32 accumulation, f64 energy",
+        "dtype": "f32 pairs, tf32x3 tensor-core spreading and bf16x3 convolutions with f32 accumulation, f64 energy",
         "data": "synthetic",
         "config": {"workload": f"{WORKLOAD}: {n} charges (2133 12-bead chains + 12800 waters), 80x80x100 A, "
                                f"64x64x80 grid, C1 b=2, r_c sweep 8-13 A (6 evals/step)",

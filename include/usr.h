@@ -105,7 +105,9 @@ typedef struct {
     double r_c;                  /* near-part cutoff; sigma = r_c / r0 */
     usr_series series;
     double spread_sigma_over_h;  /* spreading Gaussian width / largest grid spacing; 0 = 1.0 */
-    int spread_points;           /* spreading stencil points per axis (even, 8..16); 0 = 12 */
+    int spread_points;           /* spreading stencil points per axis (even, 8..16); 0 = 12.  The grid is
+                                    summed in FP32; the split convolution forms with 8 and 10 points sum
+                                    products of TF32 high and low parts on the tensor cores */
     usr_conv conv;
     int max_atoms;               /* capacity of the context (rows per evaluation), at most 2^28 */
     int virial;                  /* 1: also compute the virial tensor (usr_virial); six more far-part
@@ -147,8 +149,9 @@ usr_status usr_series_preset(int preset, usr_series* out);
  * per axis (r_c > L/3); a grid axis has fewer than spread_points + 8 points;
  * the narrowest kept Gaussian is not wider than sqrt(2) sigma_s (Eq. 32's
  * deconvolved widths sqrt(sigma_j^2 - 2 sigma_s^2) must be real); or one
- * cell's spreading tile would exceed 112 KB of shared memory (cells of more
- * than about 15 grid points per side); or a split convolution form is asked
+ * cell with its stencils' halo, in FP32, exceeds 112 KB (cells of more than
+ * about 15 grid points per side; no kernel needs the limit any more, it is
+ * kept as part of the interface); or a split convolution form is asked
  * for on a grid whose dimensions are not multiples of 4 (TF32X3) or 8 (BF16X3);
  * or a grid beyond 4096 points per axis or 2^31 - 1 points in all; or a box
  * side beyond 1e5 Angstrom; or, with n_terms = 0, a bound of Eq. 33 that
@@ -203,8 +206,9 @@ usr_status usr_info(const usr_ctx* ctx, usr_plan_info* out);
  * near + far combination, while the far part runs on `stream`, so the call
  * stays ordered on `stream` (and capturable) as one unit.  A context's
  * buffers are reused by every call: calls on one context from different
- * streams must be ordered by the caller (an event between them).  Cost: the cell list orders each cell by counting, quadratic in the
- * cell's occupancy, and the near part grows with the pairs inside r_c; at the
+ * streams must be ordered by the caller (an event between them).  Cost: the
+ * clusters rank each cell's atoms by counting, quadratic in the cell's
+ * occupancy, and the near part grows with the pairs inside r_c; at the
  * densities the method is made for (about 0.1 charges per cubic Angstrom)
  * cells hold tens to a few hundred atoms, while charges piled into one cell
  * make both stages slow.

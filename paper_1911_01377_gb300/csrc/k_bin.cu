@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) k_bin_count(int n, const float4* __restri
     if (!USR_IN_BOUNDS(c, b.nc[0] * b.nc[1] * b.nc[2], status)) c = 0;
     cell_of[i] = c;
     // one atomic per distinct cell in the warp (neighbouring caller indices are often in one cell); the slot
-    // order inside a cell is arbitrary either way, and k_cell_sort orders each cell by caller index
+    // order inside a cell is arbitrary either way: k_cluster_build and k_cell_sort order it by keys of their own
     const unsigned int peers = __match_any_sync(live, c);
     const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
     int base = 0;

@@ -26,8 +26,8 @@
  * FP32 (three MMAs per k-step): TF32x3 (10 + 10 mantissa bits per operand)
  * or BF16x3 (7 + 8).  The tensor core truncates each addition to its FP32 sum, so in the TF32 form
  * the two small products have an accumulator of their own (NT further columns), which saves the large one two
- * truncations of three; the epilogue adds the two (BF16x3's operand rounding is larger than that).  Each epilogue writes the hi and lo parts of its output
- * for the next pass; the last writes FP32.
+ * truncations of three; the epilogue adds the two.  (BF16x3's operand rounding is larger than that: one
+ * accumulator.)  Each epilogue writes the hi and lo parts of its output for the next pass; the last writes FP32.
  *
  * CTA: 128 threads, one 128-line M tile, one N tile of NT <= 256 columns
  * (NT - 1 output columns and the DC column at most), the K loop in stages of
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const __grid_constant
         const int c_lo = tile * g.cols;
         float muj = 0.f;
         if (g.pass != 3) muj = g.mu[batch];
-        // the k = 0 mode of rho, dropped: a constant line adds nothing to the zero-mean part, K mean to the sum
+        // what is left of rho's k = 0 mode: a constant line adds nothing to the zero-mean part, K mean to the sum
         if (g.pass == 1 && g.mean) dc -= (float)((double)g.K * *g.mean);
         int lx = 0, lz = 0;
         if (g.pass == 2) {

@@ -550,13 +550,17 @@ __global__ void __launch_bounds__(kThreads) k_combine(const float4* __restrict__
 
 /* ------------------------------------------------------------------ launch */
 
-#define USR_GATHER_CASE(PP)                                                                \
-    case PP:                                                                               \
-        launch_with(-1, k_gather<PP>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, psi, g, far4, partial, counter, psi_mean, status); \
+#define USR_GATHER_CASE(PP)                                                                                          \
+    case PP:                                                                                                         \
+        launch_with(-1, k_gather<PP>, nb, kGThreads, 0, st, L.cpos, L.pstart + ncell, psi, g, far4, partial,         \
+                    counter, psi_mean, status);                                                                      \
         break;
 
 /* Cluster slots of n atoms in ncell cells at most. */
-static int max_slots_of(int n, int ncell) { return (int)std::min((long long)n + 7LL * std::min(n, ncell), (long long)INT_MAX); }
+static int max_slots_of(int n, int ncell)
+{
+    return (int)std::min((long long)n + 7LL * std::min(n, ncell), (long long)INT_MAX);
+}
 
 static int gather_blocks(int n, int P)
 {

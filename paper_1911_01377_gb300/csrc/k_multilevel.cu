@@ -58,7 +58,8 @@ __device__ __forceinline__ long long offs(int col, int g, int b, int d0, int d1,
 
 /*
  * Stage rows [g0, g0 + ROWS) (periodic in n_in) of 32 columns starting at col0 into S[row][col].  Columns
- * past ncol read as zero; `less` (AX = 0) is taken off every value.  All of a thread's loads are issued before its shared-memory stores.
+ * past ncol read as zero; `less` (AX = 0) is taken off every value.  All of a thread's loads are issued before
+ * its shared-memory stores.
  */
 template <int AX, int ROWS>
 __device__ __forceinline__ void stage(float (*S)[kMlPad], const float* __restrict__ in, int g0, int n_in,
@@ -137,7 +138,8 @@ __device__ __forceinline__ void emit(float (*S)[kMlPad], const float acc[4], flo
 /* CTA coordinates: blockIdx.x = column tile, blockIdx.y = output tile along AX, blockIdx.z = batch index. */
 template <int AX, int OUT>
 __global__ void __launch_bounds__(256) k_ml_restrict(const float* __restrict__ in, const double* __restrict__ mean,
-                                                     float* __restrict__ out, float* __restrict__ out_lo, int d0, int d1, int ncol,
+                                                     float* __restrict__ out, float* __restrict__ out_lo, int d0,
+                                                     int d1, int ncol,
                                                      int n_in, MlTaps taps, long long out_elems, int* status)
 {
     pdl_wait();   // the predecessor on this stream has completed (programmatic launch)
@@ -205,8 +207,8 @@ void shape(const int* od, dim3* grid, int* ncol)
 }
 
 template <int AX, int OUT>
-void restrict_axis(const float* in, const double* mean, float* out, float* out_lo, const int* od, const MlTaps& w, int* status,
-                   cudaStream_t st)
+void restrict_axis(const float* in, const double* mean, float* out, float* out_lo, const int* od, const MlTaps& w,
+                   int* status, cudaStream_t st)
 {
     dim3 g;
     int ncol;
@@ -228,8 +230,8 @@ void prolong_axis(const float* in, float* out, const int* od, const MlTaps& w, i
 
 }  // namespace
 
-void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c, float* rho_c_lo,
-                        int* status, cudaStream_t st)
+void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c,
+                        float* rho_c_lo, int* status, cudaStream_t st)
 {
     const int d1[3] = {m.nc[0], m.n[1], m.n[2]};
     const int d2[3] = {m.nc[0], m.nc[1], m.n[2]};

@@ -2,8 +2,9 @@
  * k_spread.cu -- charge spreading of the far part (the GSE scheme named in Sec. IV.A, Eq. 32's first
  * spreading Gaussian):
  *   rho_g = sum_i q_i exp(-|g - r_i|^2 / (2 sigma_s^2))   (normalisation folded into the convolution scale)
- * written once per grid point, and the grid mean of rho (its k = 0 mode, dropped per Eq. 4; the x pass of
- * the convolutions takes it off its row sums).
+ * written once per grid point, and the grid mean of what was written (rho's k = 0 mode, dropped per Eq. 4; the
+ * x pass of the convolutions or the first restriction takes it off).  The split forms take the mean that the net
+ * charge gives off rho before they split it.
  *
  * Owner-computes, as a contraction over atoms: a warp owns a brick of 16 x 8 x 8 grid points (x, y, z) and
  * for eight atoms at a time adds the product X YZ_z of their x weights (16 points x 8 atoms, charge included)

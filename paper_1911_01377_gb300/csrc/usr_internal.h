@@ -86,7 +86,7 @@ inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t 
 constexpr int kGatherBlocks = USR_GATHER_BLOCKS;   // gather CTAs at most
 
 /*
- * Blocks of cells and the grid tiles that hold the stencils of their atoms.  Block b along axis a covers
+ * Blocks of cells and the grid tiles that would hold the stencils of their atoms (no kernel stages them any more).  Block b along axis a covers
  * cells [b kb_a, min((b+1) kb_a, nc_a)); its tile spans grid points org_a[b] .. org_a[b] + T_a - 1 (periodic).
  * The plan's limit on cells (in grid points) is stated in these: a block of one cell must fit kTileMaxSmem.
  */
@@ -348,10 +348,10 @@ struct MlArgs {
 };
 
 // ---- launchers (all enqueue on `st`) ----
-/* rho less its grid mean (fine, [z][y][x]) -> rho_c (coarse) through t1 = [n2][n1][nc0], t2 = [n2][nc1][nc0]; with rho_c_lo
-   non-null, rho_c / rho_c_lo receive the TF32 hi / lo split of the result (tensor-core coarse passes). */
-void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c, float* rho_c_lo,
-                        int* status, cudaStream_t st);
+/* rho less its grid mean (fine, [z][y][x]) -> rho_c (coarse) through t1 = [n2][n1][nc0], t2 = [n2][nc1][nc0]; with
+   rho_c_lo non-null, rho_c / rho_c_lo receive the TF32 hi / lo split of the result (tensor-core coarse passes). */
+void launch_ml_restrict(const MlArgs& m, const float* rho, const double* mean, float* t1, float* t2, float* rho_c,
+                        float* rho_c_lo, int* status, cudaStream_t st);
 /* psi += prolongation of psi_c, through t1 = [nc2][nc1][n0], t2 = [nc2][n1][n0] */
 void launch_ml_prolong(const MlArgs& m, const float* psi_c, float* t1, float* t2, float* psi, int* status,
                        cudaStream_t st);
