@@ -354,8 +354,9 @@ __global__ void __launch_bounds__(kGThreads, (P <= 10 ? USR_GATHER_MINB : 2) * 2
  * independent, then its x points and rows; the warp sums the lanes at the end.  The z weights come from
  * shared memory (lane k evaluates weight k), the x and y weights are the lane's own.
  *
- * Bound: L1 wavefronts (the rows of a load fall on overlapping banks).  A row is one two-wide load where k_gather
- * spreads each load over 8 atoms' rows: alone on the slab (12 points) 90 -> 76 us.  With 10 points the two are
+ * Bound: L1 wavefronts (68 % of their peak on the slab; k_gather 56 % at 8 points there and 81 % at 10 for 200 k
+ * charges): the rows of a load fall on overlapping banks.  A row is one two-wide load where k_gather spreads each
+ * load over 8 atoms' rows: alone on the slab (12 points) 90 -> 76 us.  With 10 points the two are
  * equal (130 against 124 us for 200 k charges) and with 8, four points to a lane, this form is slower (44 against
  * 35 us on the slab): the weights then cost more than the rows.
  */

@@ -32,8 +32,8 @@
  * candidates (all its cells together) are tested 32 at a time, the next surviving j-cluster's atoms are loaded
  * while the current one's steps run, and the next unit is taken from the queue during the current one.
  *
- * Bound: issue slots and the latency of the step's chain (55 % of the slots used at 16 warps per SM; about 105
- * instructions per step that has a pair inside r_c, 32 of them two-wide FP32).  Alone, slab at r_c = 8 / 10 / 13 A:
+ * Bound: issue slots and the latency of the step's chain (57 to 61 % of the slots used at 16 warps per SM; FMA pipe
+ * 20 to 23 %, L1 28 to 33 %).  Alone, slab at r_c = 8 / 10 / 13 A:
  * 76 / 98 / 179 us, 200 k charges at 9 A 246 us, 1.06 M at 10 A 1.44 ms, against 92 / 126 / 212 us, 305 us and 1.75
  * ms with i atoms in registers, clusters in Morton order and one scan per neighbour cell.  Not kept: constants
  * pinned in registers (no change: the instructions take them from constant memory); the surviving clusters as a

@@ -34,16 +34,18 @@
  * S-th chunk of the list, and their sums are added in a fixed order at the end.  There are no atomics, no
  * halo and no second pass over tiles, and every point receives its terms in a fixed order.
  *
- * Bound: issue slots (about 45 % of them used) and the latency of the list.  (P + 15) / 16 ((P + 7) / 8)^2
- * bricks per atom at about 25 instructions each, and one to two per atom listed.  Alone (ncu): 42 us on the
- * slab at r_c = 8 A (P = 8), 111 us for 200 k charges (P = 10).  The earlier form (shared-memory tiles per
- * block of cells, one read-modify-write per stencil point, then a reduction over overlapping tiles) took
- * 36 + 23 us and 157 + 73 us: 940 instructions per atom at P = 10 against 290, held by shared-memory
- * wavefronts and by the tiles' 13-fold halo traffic.  Bricks summed by FP32 FMAs instead took 217 us (the
- * register side of broadcast loads), this contraction with weight rows shared by a CTA's warps 172 us
- * (barriers).  Not kept either: the sums by two-wide FP32 FMAs of each warp (evaluations 1 to 3 % slower, the
- * FP32 pipe is the pair kernel's); up to 16 warps per brick on one flattened list (68 -> 65 us per evaluation of
- * 2 k charges, 598 -> 606 us of 200 k).
+ * Bound: issue slots and the latency of the list (39 % of the slots used on the slab, whose 320 bricks leave two warps
+ * to a scheduler, 59 % for 200 k charges; tensor pipe 21 and 32 % active).  (P + 15) / 16 ((P + 7) / 8)^2 bricks per
+ * atom at 44 instructions each, the listing included.  Alone (ncu): 42 us on the slab at r_c = 8 A (P = 8), 115 us
+ * for 200 k charges (P = 10), 328 us for 1.06 M (P = 8); FMA form 71 us on the slab (P = 12; 52 % of the slots).
+ * The earlier form (shared-memory tiles per block of cells, one read-modify-write per stencil point, then a reduction
+ * over overlapping tiles) took 36 + 23 us and 157 + 73 us (141 at P = 12): 940 instructions per atom at P = 10
+ * against 310, held by shared-memory wavefronts and by the tiles' 13-fold halo traffic.  Not kept: bricks of a CTA
+ * with weight rows shared by its warps, by FP32 FMAs 217 us (the register side of broadcast loads), on the tensor
+ * cores 172 us (barriers); FMAs where the stencil does not need them (evaluations of the split forms 1 to 3 % slower,
+ * the FP32 pipe is the pair kernel's); the tensor cores with compensated sums of the groups in the FP32 form (the
+ * drop's far potential off by 5.7e-6, slab 280 us per evaluation); up to 16 warps per brick on one flattened list
+ * (68 -> 65 us per evaluation of 2 k charges, 598 -> 606 us of 200 k).
  */
 #include <algorithm>
 
